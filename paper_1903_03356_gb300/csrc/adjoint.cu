@@ -1210,6 +1210,16 @@ lbmib_status tape_forward(lbmib_ctx* c, lbmib_scheme scheme, int len, char* w, c
     double2* tX = (double2*)(w + a.tape_X);
     LBMIB_CUDA(c, cudaMemcpyAsync(tape, c->pops[c->cur], pbytes, cudaMemcpyDeviceToDevice, s));
     LBMIB_CUDA(c, cudaMemcpyAsync(w + a.age0, c->nd.age, M * sizeof(int), cudaMemcpyDeviceToDevice, s));
+    if (wide(c)) {
+        const WideTape t{tape, a.pb, M, tX, scheme == LBMIB_DYNAMIC ? (double2*)(w + a.tape_flc) : nullptr};
+        LBMIB_CUDA(c, cudaMemcpyAsync(tX, c->nd.X, M * sizeof(double2), cudaMemcpyDeviceToDevice, s));
+        int cur = 0;
+        enqueue_wide(c, scheme, len, cur, c->cur_fib, s, &t);
+        LBMIB_CUDA(c, cudaMemcpyAsync(c->pops[c->cur], tape + (size_t)len * a.pb, pbytes, cudaMemcpyDeviceToDevice, s));
+        LBMIB_CUDA(c, cudaGetLastError());
+        c->steps += len;
+        return LBMIB_OK;
+    }
     void* keep0 = c->pops[0];
     void* keep1 = c->pops[1];
     fork_ib(c, s);

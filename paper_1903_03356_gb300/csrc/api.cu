@@ -154,6 +154,72 @@ void with_ib_storage(const lbmib_ctx* c, F&& f) {
 // (k_dyn_update_spread): one CTA per capsule and no rigid particles.
 bool fusable(const lbmib_ctx* c) { return c->fuse_ib && c->arcs == 1 && c->nrigid == 0 && !c->caps.empty(); }
 
+// Whether steps run as two kernels each (wide.cu): few capsules on a lattice that stays in
+// L2, with every option that asks for the other kernels at its default. Lines:
+//  - up to kWideNodes the force field read in place costs less than the patch (its launch,
+//    list and claims);
+//  - up to kWideVerts vertices (a quarter of that where the interpolations are in FP64, whose
+//    pipe the nine-lane gathers would fill) the gathers of every support node are cheaper
+//    than the tiles' chain;
+//  - in single precision only where a tiled arc is longer than a warp: shorter arcs add
+//    their float shares in a fixed order, so that a tiled run repeats bit for bit, and
+//    positions, which add up every step's rounding, would part from it by 1e-9 in 200 steps.
+bool wide(const lbmib_ctx* c) {
+    constexpr long long kWideNodes = 1 << 20, kWideVerts = 32768;
+    const bool fp64 = c->cfg.storage == LBMIB_FP64 || c->ib_fp64;
+    if (c->caps.empty() || c->nrigid > 0 || !c->fuse_ib || c->timing || c->overlap != -1 || c->arcs_opt != 0)
+        return false;
+    if (!fp64 && (c->max_n + c->arcs - 1) / c->arcs <= 32) return false;
+    return (long long)c->cfg.nx * c->cfg.ny <= kWideNodes && c->nd.count <= (fp64 ? kWideVerts / 4 : kWideVerts) &&
+           wide_fits(c->max_n, wide_arcs(c->max_n, (int)c->caps.size(), c->sms > 0 ? c->sms : 1));
+}
+
+// Enqueue n steps of one scheme on stream s in the two-kernel form:
+//   spread | lattice + force, update + next spread | ... | lattice + force, update
+// With `tape`, step k reads and writes population buffers k and k + 1 of the tape and the
+// positions after it and the c_l F_l of its spread go to the tape's slots.
+void enqueue_wide(lbmib_ctx* c, lbmib_scheme scheme, long long n, int& cur, int& cur_fib, cudaStream_t s,
+                  const WideTape* tape) {
+    const int ncaps = (int)c->caps.size();
+    const int arcs = wide_arcs(c->max_n, ncaps, c->sms > 0 ? c->sms : 1);
+    const bool dyn = scheme == LBMIB_DYNAMIC, rep = ncaps > 1 && c->rep_rc > 0.0;
+    const int cap = 9 * (c->cfg.max_nodes > 0 ? c->cfg.max_nodes : 1);
+    unsigned* status = &c->ctr->status;
+    const Lat& L = c->L;
+    Nodes nd = c->nd;
+    bool spread_done = false;
+    for (long long k = 0; k < n; k++) {
+        const void* src = tape ? (const void*)(tape->pops + (size_t)k * tape->stride) : c->pops[cur];
+        void* dst = tape ? (void*)(tape->pops + (size_t)(k + 1) * tape->stride) : c->pops[1 - cur];
+        const int fc = 1 - cur_fib, fp = cur_fib;
+        if (rep) {
+            launch_repulsion(L, nd, ncaps, c->max_n, c->arcs, c->rep, status, s);
+            c->launches += 2;
+        }
+        auto ib = [&](bool upd, bool spr, const void* pops, int to, double2* tape_x, bool pdl) {
+            with_ib_storage(c, [&](auto v) {
+                launch_wide<decltype(v)>(dyn, upd, spr, pops, L, nd, ncaps, c->max_n, arcs, c->fib[fc], c->fib[to],
+                                         c->list[to], &c->ctr->count[to], status, tape_x, pdl, s);
+            });
+            c->launches++;
+        };
+        if (!spread_done) {
+            nd.Flc = tape && tape->flc ? tape->flc + k * tape->nodes : nullptr;
+            ib(false, true, src, fc, nullptr, false);
+        }
+        by_storage(c->cfg.storage, [&](auto tag) {
+            launch_collide_forced<decltype(tag)>(src, dst, L, c->open, c->fib[fc], c->fib[fp], c->list[fp],
+                                                 &c->ctr->count[fp], cap, status, true, s);
+        });
+        c->launches++;
+        spread_done = k + 1 < n && (dyn || !rep);   // the Kinematic spread needs the repulsion at X^{n+1}
+        nd.Flc = tape && tape->flc && spread_done ? tape->flc + (k + 1) * tape->nodes : nullptr;
+        ib(true, spread_done, dst, fp, tape ? tape->X + (k + 1) * tape->nodes : nullptr, true);
+        cur_fib = fc;
+        cur = 1 - cur;
+    }
+}
+
 // Enqueue one coupled step on stream s, advancing (cur, cur_fib). `spread_done`: the
 // previous step's update already did this step's force and spread; `fuse_next`: another
 // step of the same scheme follows in this run, so the update may do its force and
@@ -301,6 +367,10 @@ bool enqueue_step(lbmib_ctx* c, lbmib_scheme scheme, int& cur, int& cur_fib, cud
 // Enqueue n steps of one scheme on stream s, fusing each Dynamic update with the next
 // step's force and spread where fusable.
 void enqueue_steps(lbmib_ctx* c, lbmib_scheme scheme, long long n, int& cur, int& cur_fib, cudaStream_t s, bool timed) {
+    if (wide(c)) {
+        enqueue_wide(c, scheme, n, cur, cur_fib, s, nullptr);
+        return;
+    }
     bool ahead = false;
     for (long long k = 0; k < n; k++) ahead = enqueue_step(c, scheme, cur, cur_fib, s, timed, ahead, k + 1 < n);
 }
@@ -353,6 +423,7 @@ void update_arcs(lbmib_ctx* c) {
     c->max_arc_len = arc;
     c->tile_cells = cells;
     set_capsule_smem_limits(slots, cells);
+    set_wide_smem_limits(std::max(c->max_n, 1), wide_arcs(std::max(c->max_n, 1), ncaps, c->sms > 0 ? c->sms : 1));
     drop_graphs(c);   // launch shapes may have changed
 }
 

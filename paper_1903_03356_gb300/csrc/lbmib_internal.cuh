@@ -202,7 +202,7 @@ __device__ __forceinline__ void open_column(C (&s)[9], const Lat& L, const OpenB
 // and every load issued before any is used, and, given the open-channel data ob, the
 // Zou-He closure on the open columns. NC as for pull().
 template <typename S, bool NC = true>
-__device__ __forceinline__ void pull_all(const S* __restrict__ src, const Lat& L, int x, int y,
+__device__ __forceinline__ void pull_all(const S* src, const Lat& L, int x, int y,
                                          typename St<S>::C (&s)[9], const OpenBC* ob = nullptr) {
     using C = typename St<S>::C;
     const int xm = x == 0 ? L.nx - 1 : x - 1, xp = x + 1 == L.nx ? 0 : x + 1;
@@ -614,12 +614,12 @@ struct Mom {
     C drho, ux, uy;
 };
 
-template <typename S>
-__device__ __forceinline__ Mom<typename St<S>::C> node_moments(const S* __restrict__ src, const Lat& L,
-                                                               const double* __restrict__ fib, int x, int y) {
+template <typename S, bool NC = true>
+__device__ __forceinline__ Mom<typename St<S>::C> node_moments(const S* src, const Lat& L, const double* fib, int x,
+                                                               int y) {
     using C = typename St<S>::C;
     C s[9];
-    pull_all<S>(src, L, x, y, s);
+    pull_all<S, NC>(src, L, x, y, s);
     C drho, mx, my;
     moments<C>(s, drho, mx, my);
     const long long N = (long long)L.nx * L.ny;

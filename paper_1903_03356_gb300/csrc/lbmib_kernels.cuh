@@ -115,6 +115,24 @@ void launch_observables(Nodes nd, int ncaps, int max_n, double* out, cudaStream_
 template <typename S>
 void launch_interp_points(const void* src, const Lat& L, const double* fib, const double2* pts, int n,
                           double* out, unsigned* status, cudaStream_t s);
+// wide.cu: the two-kernel step of few capsules on a lattice in L2. `arcs` CTAs per capsule
+// (a cluster); upd: node update on the state `pops` of step n (Kinematic: with half of the
+// force fib_n), spr: force and spread of the next step into fib and its list; count: the
+// list's length (0 without a spread); tape (may be null): X^{n+1} of every vertex; pdl:
+// may start before the kernel before it has finished (that kernel writes no vertex data).
+int wide_arcs(int max_n, int ncaps, int sms);
+bool wide_fits(int max_n, int arcs);   // the arcs' staged vertices fit the shared memory of a CTA
+void set_wide_smem_limits(int max_n, int arcs);
+template <typename S>
+void launch_wide(bool dynamic, bool upd, bool spr, const void* pops, const Lat& L, Nodes nd, int ncaps, int max_n,
+                 int arcs, const double* fib_n, double* fib, int* list, int* count, unsigned* status, double2* tape,
+                 bool pdl, cudaStream_t s);
+// lattice update with the force field `fib` (and the open columns), clearing fib_p at its
+// listed nodes
+template <typename S>
+void launch_collide_forced(const void* src, void* dst, const Lat& L, const OpenBC& ob, const double* fib,
+                           double* fib_p, const int* list_p, const int* count_p, int capacity, unsigned* status,
+                           bool pdl, cudaStream_t s);
 // repulsion.cu
 void launch_repulsion(const Lat& L, Nodes nd, int ncaps, int max_n, int arcs, RepGrid g, unsigned* status,
                       cudaStream_t s);
