@@ -231,6 +231,57 @@ __global__ void __launch_bounds__(BS, MINB) k_collide_stream(const S* __restrict
     if (__any_sync(0xffffffffu, bad && active) && lane == 0) atomicOr(status, kStatUnstable);
 }
 
+// FP64 storage: the same loads and stores with the uniform force's constants from the host
+// (collide_d). The stability test compares the bits of u^2 (a double comparison would be one
+// more FP64 instruction).
+template <int BS, int MINB>
+__global__ void __launch_bounds__(BS, MINB) k_collide_stream_d(const double* __restrict__ src,
+                                                               double* __restrict__ dst, Lat L, CollideD k,
+                                                               unsigned* __restrict__ status) {
+    constexpr int V = 2;
+    const int lane = threadIdx.x & 31;
+    const long long gw = ((long long)blockIdx.x * BS + threadIdx.x) >> 5;
+    const int segs = (L.nx + 32 * V - 1) / (32 * V);
+    if (gw >= (long long)segs * L.ny) return;  // whole warps only
+    const int y = (int)(gw / segs);
+    const int seg = (int)(gw - (long long)y * segs);
+    const int x0 = (seg * 32 + lane) * V;
+    const bool active = x0 < L.nx, full = x0 + V <= L.nx;
+    PopLoad<double, 0, 0> p0; PopLoad<double, 1, 0> p1; PopLoad<double, 2, 0> p2;
+    PopLoad<double, 3, 0> p3; PopLoad<double, 4, 0> p4; PopLoad<double, 5, 0> p5;
+    PopLoad<double, 6, 0> p6; PopLoad<double, 7, 0> p7; PopLoad<double, 8, 0> p8;
+    p0.issue(src, L, x0, y, lane, active); p1.issue(src, L, x0, y, lane, active);
+    p2.issue(src, L, x0, y, lane, active); p3.issue(src, L, x0, y, lane, active);
+    p4.issue(src, L, x0, y, lane, active); p5.issue(src, L, x0, y, lane, active);
+    p6.issue(src, L, x0, y, lane, active); p7.issue(src, L, x0, y, lane, active);
+    p8.issue(src, L, x0, y, lane, active);
+    double f[9][V];
+    p0.resolve(src, L, x0, y, lane, active, full, f[0]); p1.resolve(src, L, x0, y, lane, active, full, f[1]);
+    p2.resolve(src, L, x0, y, lane, active, full, f[2]); p3.resolve(src, L, x0, y, lane, active, full, f[3]);
+    p4.resolve(src, L, x0, y, lane, active, full, f[4]); p5.resolve(src, L, x0, y, lane, active, full, f[5]);
+    p6.resolve(src, L, x0, y, lane, active, full, f[6]); p7.resolve(src, L, x0, y, lane, active, full, f[7]);
+    p8.resolve(src, L, x0, y, lane, active, full, f[8]);
+    bool bad = false;
+#pragma unroll
+    for (int j = 0; j < V; j++) {
+        double s[9];
+#pragma unroll
+        for (int i = 0; i < 9; i++) s[i] = f[i][j];
+        // |u| > 0.3 or NaN: non-negative doubles order as their bits, NaNs above them
+        bad |= (unsigned long long)__double_as_longlong(collide_d(s, k)) >=
+               (unsigned long long)__double_as_longlong(0.09);
+#pragma unroll
+        for (int i = 0; i < 9; i++) f[i][j] = s[i];
+    }
+    double* o = dst + (long long)y * L.pitch + x0;
+#pragma unroll
+    for (int i = 0; i < 9; i++) {
+        if (full) *reinterpret_cast<double2*>(o + (long long)i * L.plane) = make_double2(f[i][0], f[i][1]);
+        else if (active) o[(long long)i * L.plane] = f[i][0];
+    }
+    if (__any_sync(0xffffffffu, bad && active) && lane == 0) atomicOr(status, kStatUnstable);
+}
+
 // FP16 storage: one warp owns 256 consecutive nodes of a row, 8 per thread, each
 // population fetched with one aligned 16-byte load and kept packed (four half2
 // registers) until its node pair is collided; the results are packed back and stored
@@ -631,10 +682,17 @@ void launch_collide_stream(const void* src, void* dst, const Lat& L, unsigned* s
             return;
         }
     }
+    if constexpr (std::is_same<S, double>::value) {
+        const CollideD k(L.gx, L.gy, L.omega);
+        if (bs == 256) k_collide_stream_d<256, 3><<<g, 256, 0, s>>>(a, b, L, k, status);
+        else k_collide_stream_d<128, 6><<<g, 128, 0, s>>>(a, b, L, k, status);
+        return;
+    } else {
     if (bs == 256 && !occ4) k_collide_stream<S, 0, 0, 256, 3><<<g, 256, 0, s>>>(a, b, L, status);
     else if (bs == 256) k_collide_stream<S, 0, 0, 256, 4><<<g, 256, 0, s>>>(a, b, L, status);
     else if (!occ4) k_collide_stream<S, 0, 0, 128, 6><<<g, 128, 0, s>>>(a, b, L, status);
     else k_collide_stream<S, 0, 0, 128, 8><<<g, 128, 0, s>>>(a, b, L, status);
+    }
 }
 
 template <typename S>

@@ -665,7 +665,7 @@ template <typename S>
 __global__ void __launch_bounds__(128) k_collide_forced(const S* src, S* dst, Lat L,
                                                         OpenBC ob, const double* fib, double* fib_p,
                                                         const int* list_p, const int* count_p, int capacity,
-                                                        unsigned* status) {
+                                                        CollideD kd, unsigned* status) {
     using C = typename St<S>::C;
     const long long N = (long long)L.nx * L.ny;
     const int node = blockIdx.x * blockDim.x + threadIdx.x;
@@ -683,7 +683,14 @@ __global__ void __launch_bounds__(128) k_collide_forced(const S* src, S* dst, La
             Fx = C(L.gx + __longlong_as_double(bx));
             Fy = C(L.gy + __longlong_as_double(by));
         }
-        const C usq = collide<C>(s, Fx, Fy, lat_c<C>(L.omega, L.omegaf));
+        C usq;
+        if constexpr (sizeof(C) == 8) {   // the uniform force's constants come from the host
+            CollideD k = kd;
+            if (((bx | by) << 1) != 0) k = CollideD(Fx, Fy, L.omega);
+            usq = collide_d(s, k);
+        } else {
+            usq = collide<C>(s, Fx, Fy, L.omegaf);
+        }
         bad = !(usq < C(0.09));   // |u| > 0.3 or NaN
         S* o = dst + (long long)y * L.pitch + x;
 #pragma unroll
@@ -798,7 +805,7 @@ void launch_collide_forced(const void* src, void* dst, const Lat& L, const OpenB
     const long long N = (long long)L.nx * L.ny;
     const int bs = sizeof(typename St<S>::C) == 8 ? 64 : 128;
     launch_pdl(&k_collide_forced<S>, dim3((unsigned)((N + bs - 1) / bs)), bs, 0, 1, pdl, s, (const S*)src, (S*)dst, L,
-               ob, fib, fib_p, list_p, count_p, capacity, status);
+               ob, fib, fib_p, list_p, count_p, capacity, CollideD(L.gx, L.gy, L.omega), status);
 }
 
 #define LBMIB_INSTANTIATE_WIDE(S)                                                                              \
