@@ -614,12 +614,27 @@ __device__ __forceinline__ MlsW<C> mls_weights(int cx, int cy, C d0x, C d0y, boo
     m.ok = ok;
     m.sane = true;
     C dx[3], dy[3], sx0 = 0, sx1 = 0, sy0 = 0, sy1 = 0;
+    if constexpr (sizeof(C) == 8) {
+        // The fit does not change when an axis's weights share a factor: with w_0 = 1,
+        // w_a = exp(-c) exp(-2 a d0 c), one exponential (some twenty FP64 instructions) and one
+        // reciprocal per axis instead of three exponentials (4096 x 512 channel with 256
+        // capsules, FP64: 412 -> 402 us per step).
+        constexpr double kExpC = 0.19327224468471937;   // exp(-1 / (r_w alpha)^2)
+        const double X = exp(-2.0 * kMlsInvLen2 * d0x), Y = exp(-2.0 * kMlsInvLen2 * d0y);
+        m.wx[0] = kExpC * rcp_newton(X);
+        m.wy[0] = kExpC * rcp_newton(Y);
+        m.wx[1] = m.wy[1] = 1.0;
+        m.wx[2] = kExpC * X;
+        m.wy[2] = kExpC * Y;
+    }
 #pragma unroll
     for (int a = 0; a < 3; a++) {
         dx[a] = d0x + C(a - 1);
         dy[a] = d0y + C(a - 1);
-        m.wx[a] = exp(-dx[a] * dx[a] * C(kMlsInvLen2));
-        m.wy[a] = exp(-dy[a] * dy[a] * C(kMlsInvLen2));
+        if constexpr (sizeof(C) == 4) {
+            m.wx[a] = exp(-dx[a] * dx[a] * C(kMlsInvLen2));
+            m.wy[a] = exp(-dy[a] * dy[a] * C(kMlsInvLen2));
+        }
         sx0 += m.wx[a];
         sx1 += m.wx[a] * dx[a];
         sy0 += m.wy[a];
