@@ -458,8 +458,9 @@ __global__ void __launch_bounds__(128) k_ragged_h(const __half* __restrict__ src
 // patch reads and writes each node's own nine slots and nothing else of the lattice. A
 // node that several capsules' tiles cover is listed more than once: the first thread to
 // claim it (an atomic exchange of this launch's stamp, issued with the loads) patches it,
-// the others leave it. The last block to finish advances the stamp. Also clears the
-// previous force buffer at the previous list (its last reader has run).
+// the others leave it. The last block to finish advances the stamp and empties the previous
+// list, to which the next spread appends. Also clears the previous force buffer at the
+// previous list (its last reader has run).
 template <typename S>
 __global__ void __launch_bounds__(256) k_patch(S* __restrict__ dst, Lat L, const double* __restrict__ fib_c,
                                                const int* __restrict__ list_c, double* __restrict__ fib_p,
@@ -527,6 +528,7 @@ __global__ void __launch_bounds__(256) k_patch(S* __restrict__ dst, Lat L, const
         __threadfence();
         if (atomicAdd(&ctr->patch_blocks, 1) == (int)gridDim.x - 1) {
             ctr->patch_blocks = 0;
+            ctr->count[1 - c] = 0;   // every block has read it; the next spread appends from here
             ctr->step_stamp = stamp;
         }
     }
