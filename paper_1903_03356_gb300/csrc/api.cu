@@ -66,9 +66,11 @@ Layout make_layout(const lbmib_config* c) {
     L.Fpp = take(M * sizeof(double2));
     L.rep_buckets = 64;
     while (L.rep_buckets < 4 * (int)K) L.rep_buckets *= 2;
-    L.rep_box = take(4 * K * sizeof(double));
+    L.rep_box = take(K * sizeof(float4));
+    L.rep_xf = take(M * sizeof(float2));
+    L.rep_cbox = take((M / 32 + K + 1) * sizeof(float4));
     L.rep_cellof = take(K * sizeof(int));
-    L.rep_count = take((size_t)L.rep_buckets * sizeof(int));
+    L.rep_count = take(((size_t)L.rep_buckets + 1) * sizeof(int));
     L.rep_slot = take((size_t)L.rep_buckets * kRepSlots * sizeof(int));
     L.pts = take(M * sizeof(double2));
     L.pts_out = take(8 * M * sizeof(double));
@@ -104,12 +106,12 @@ void drop_graphs(lbmib_ctx* c) {
                 }
 }
 
-// Stream schedule of one step (FS force+spread, CS collide-stream, P patch, U update):
-//   ib stream:      FS(n) ----------+                 +--> U(n) --> FS(n+1) ...
 // Whether the Dynamic node update of a step may also do the force and spread of the next
 // (k_dyn_update_spread): one CTA per capsule and no rigid particles.
 bool fusable(const lbmib_ctx* c) { return c->fuse_ib && c->arcs == 1 && c->nrigid == 0 && !c->caps.empty(); }
 
+// Stream schedule of one step (FS force+spread, CS collide-stream, P patch, U update):
+//   ib stream:      FS(n) ----------+                 +--> U(n) --> FS(n+1) ...
 //   lattice stream: CS(n) ------- wait --> P(n) --+---+--> CS(n+1) ...
 // CS reads only the populations and the uniform force, so it does not wait for FS; P
 // needs both. CS(n+1) needs the patched populations only, so it runs beside U(n) and
@@ -120,14 +122,14 @@ bool fusable(const lbmib_ctx* c) { return c->fuse_ib && c->arcs == 1 && c->nrigi
 // capsules to fill the GPU the IB blocks take registers and warp slots from the lattice
 // kernel, which slows by what the overlap saves. Hence the automatic setting: overlap
 // while the capsules number fewer than two per SM.
-bool overlapped(const lbmib_ctx* c) {
-    if (c->caps.empty() || c->overlap == 0) return false;
 // With FP16 storage the fused IB kernels keep the context stream: beside the lattice kernel
 // their warps add the force shares in another order from run to run, and FP16 rounding turns
 // a last-place difference into a thousandth of a population.
+bool overlapped(const lbmib_ctx* c) {
+    if (c->caps.empty() || c->overlap == 0) return false;
+    if (c->overlap == -1 && c->cfg.storage == LBMIB_FP16 && fusable(c)) return false;
     return c->overlap == 1 || (int)c->caps.size() < 2 * (c->sms > 0 ? c->sms : 1);
 }
-    if (c->overlap == -1 && c->cfg.storage == LBMIB_FP16 && fusable(c)) return false;
 
 void fork_ib(lbmib_ctx* c, cudaStream_t s) {
     if (!overlapped(c)) return;
@@ -538,7 +540,9 @@ lbmib_status lbmib_create(const lbmib_config* cfg, void* d_arena, size_t arena_b
     c->rep.count = (int*)(a + lay.rep_count);
     c->rep.slot = (int*)(a + lay.rep_slot);
     c->rep.cellof = (int*)(a + lay.rep_cellof);
-    c->rep.box = (double*)(a + lay.rep_box);
+    c->rep.box = (float4*)(a + lay.rep_box);
+    c->rep.xf = (float2*)(a + lay.rep_xf);
+    c->rep.cbox = (float4*)(a + lay.rep_cbox);
     c->rep.nbuckets = lay.rep_buckets;
     c->d_caps = (CapsuleParams*)(a + lay.caps);
     c->nd.caps = c->d_caps;
@@ -594,6 +598,7 @@ lbmib_status lbmib_create(const lbmib_config* cfg, void* d_arena, size_t arena_b
     if (e == cudaSuccess) e = cudaMemsetAsync(c->fib[1], 0, 2 * N * sizeof(double), c->stream);
     if (e == cudaSuccess) e = cudaMemsetAsync(c->mark, 0, N * sizeof(int), c->stream);
     if (e == cudaSuccess) e = cudaMemsetAsync(c->ctr, 0, sizeof(DevCounters), c->stream);
+    if (e == cudaSuccess) e = cudaMemsetAsync(c->rep.count, 0, ((size_t)lay.rep_buckets + 1) * sizeof(int), c->stream);
     if (e != cudaSuccess) {
         lbmib_destroy(c);
         return LBMIB_ERR_CUDA;

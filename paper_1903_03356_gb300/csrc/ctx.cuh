@@ -22,7 +22,7 @@ inline size_t storage_bytes(lbmib_storage s) { return s == LBMIB_FP64 ? 8 : (s =
 struct Layout {
     size_t pops[2], fib[2], mark, list[2], ctr, scratch;
     size_t X, Xm1, uv, Fint, Fext, U, L0, c0, s0, age, capid, mls, caps, obs, pts, pts_out;
-    size_t Fpp, rep_box, rep_cellof, rep_count, rep_slot, u_in, rb, R0;
+    size_t Fpp, rep_box, rep_xf, rep_cbox, rep_cellof, rep_count, rep_slot, u_in, rb, R0;
     int rep_buckets;
     size_t total;
     int pitch;

@@ -44,10 +44,12 @@ struct RepGrid {
     double cellx, celly;   // coarse cell sides (>= largest capsule extent + cut-off)
     int ncx, ncy;      // coarse cells along x and y
     int nbuckets;      // power of two
-    int* count;        // per bucket (cleared every step)
+    int* count;        // per bucket, then the narrow phase's finished CTAs (zero between steps)
     int* slot;         // nbuckets x kRepSlots capsule ids
     int* cellof;       // per capsule: its coarse cell (iy * ncx + ix)
-    double* box;       // per capsule: min x, min y, max x, max y
+    float4* box;       // per capsule: min x, min y, max x, max y of the float positions
+    float2* xf;        // per vertex: the position rounded to float
+    float4* cbox;      // per 32-vertex chunk of every ring: its box
     double rc, coeff;  // cut-off and coefficient of Eq. 27
 };
 constexpr int kRepSlots = 16;

@@ -7,11 +7,16 @@
 //
 // Broad phase: each capsule's bounding box, and its coarse cell (side >= largest capsule
 // extent + r_c, so interacting capsules sit in neighbouring cells), hashed into
-// fixed-capacity buckets. Narrow phase: one CTA per arc of a ring stages the arc and,
-// for each capsule of the 3 x 3 neighbouring cells whose box comes within r_c of the
-// arc's box, stages that ring with the boxes of its 32-vertex chunks and sums the pair
-// forces over the chunks within r_c of each vertex. A capsule is accepted only from its
-// own cell, so hash collisions cannot count it twice.
+// fixed-capacity buckets. Narrow phase: one warp per 32 vertices of an arc; for each capsule
+// of the 3 x 3 neighbouring cells whose box comes within r_c of theirs it tests the boxes of
+// that ring's 32-vertex chunks (one lane each), and the vertices of the chunks that pass. A
+// capsule is accepted only from its own cell, so hash collisions cannot count it twice.
+//
+// A double instruction holds a warp for 64 cycles on GB300, so every test is made in float,
+// on positions rounded to float, with a reach that covers the rounding; only a pair that
+// passes is decided and evaluated in double, and only a vertex with a force forms its normal.
+// (In double throughout, the two kernels took 55 of the 83 us of a step with 16 rings of
+// 1000 vertices on 1200 x 450; now 12 of 39.)
 #include "ring.cuh"
 
 namespace lbmib {
@@ -26,27 +31,46 @@ __device__ __forceinline__ int bucket_of(int ix, int iy, int nb) {
     return (int)(h & (unsigned)(nb - 1));
 }
 
-// Bounding box, coarse cell and bucket entry of every capsule (one CTA per capsule).
+__device__ __forceinline__ float warp_min(float v) {
+    for (int o = 16; o > 0; o >>= 1) v = fminf(v, __shfl_xor_sync(0xffffffffu, v, o));
+    return v;
+}
+__device__ __forceinline__ float warp_max(float v) { return -warp_min(-v); }
+
+// First chunk box of a capsule: chunks of different capsules never share a slot.
+__device__ __forceinline__ int first_chunk(int cap, int off) { return off / 32 + cap; }
+
+// Float positions, chunk boxes, bounding box, coarse cell and bucket entry of every capsule
+// (one CTA per capsule, one warp per chunk).
 __global__ void __launch_bounds__(128) k_rep_bin(Lat L, Nodes nd, int max_n, RepGrid g, unsigned* status) {
-    __shared__ double red[32 * 8];
-    const int c = blockIdx.x;
+    __shared__ float4 part[4];
+    const int c = blockIdx.x, warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const CapsuleParams P = nd.caps[c];
     if (P.n < 3 || P.n > max_n) return;
-    double r[4] = {1e300, 1e300, 1e300, 1e300};   // min x, min y, -max x, -max y
-    for (int v = threadIdx.x; v < P.n; v += blockDim.x) {
-        const double2 X = nd.X[P.off + v];
-        r[0] = fmin(r[0], X.x);
-        r[1] = fmin(r[1], X.y);
-        r[2] = fmin(r[2], -X.x);
-        r[3] = fmin(r[3], -X.y);
+    const int first = first_chunk(c, P.off);
+    const float inf = __int_as_float(0x7f800000);
+    float4 b = make_float4(inf, inf, -inf, -inf);   // min x, min y, max x, max y
+    for (int v0 = 32 * warp; v0 < P.n; v0 += 128) {
+        const int v = v0 + lane;
+        const double2 X = nd.X[P.off + (v < P.n ? v : v0)];
+        const float2 f = make_float2((float)X.x, (float)X.y);
+        if (v < P.n) g.xf[P.off + v] = f;
+        const float4 q = make_float4(warp_min(f.x), warp_min(f.y), warp_max(f.x), warp_max(f.y));
+        if (lane == 0) g.cbox[first + v0 / 32] = q;
+        b = make_float4(fminf(b.x, q.x), fminf(b.y, q.y), fmaxf(b.z, q.z), fmaxf(b.w, q.w));
     }
-    block_reduce<4, true>(r, red);
+    if (lane == 0) part[warp] = b;
+    __syncthreads();
     if (threadIdx.x != 0) return;
-    const double b[4] = {r[0], r[1], -r[2], -r[3]};
-    for (int k = 0; k < 4; k++) g.box[4 * c + k] = b[k];
-    const bool sane = fabs(b[0]) < 1e9 && fabs(b[1]) < 1e9 && fabs(b[2]) < 1e9 && fabs(b[3]) < 1e9;
-    const double cx = sane ? 0.5 * (b[0] + b[2]) : 0.0, cy = sane ? 0.5 * (b[1] + b[3]) : 0.0;
-    if (!sane || b[2] - b[0] > g.cellx - g.rc || b[3] - b[1] > g.celly - g.rc) atomicOr(status, kStatGrid);
+    for (int w = 1; w < 4; w++) {
+        const float4 q = part[w];
+        b = make_float4(fminf(b.x, q.x), fminf(b.y, q.y), fmaxf(b.z, q.z), fmaxf(b.w, q.w));
+    }
+    g.box[c] = b;
+    // NaN positions are passed over by fminf and fmaxf: an all-NaN ring keeps the empty box
+    const bool sane = fabsf(b.x) < 1e9f && fabsf(b.y) < 1e9f && fabsf(b.z) < 1e9f && fabsf(b.w) < 1e9f;
+    const double cx = sane ? 0.5 * ((double)b.x + b.z) : 0.0, cy = sane ? 0.5 * ((double)b.y + b.w) : 0.0;
+    if (!sane || (double)b.z - b.x > g.cellx - g.rc || (double)b.w - b.y > g.celly - g.rc) atomicOr(status, kStatGrid);
     int ix = (int)floor(cx / g.cellx) % g.ncx;
     if (ix < 0) ix += g.ncx;
     int iy = (int)floor(cy / g.celly);
@@ -62,135 +86,118 @@ __global__ void __launch_bounds__(128) k_rep_bin(Lat L, Nodes nd, int max_n, Rep
     else atomicOr(status, kStatGrid);
 }
 
-constexpr int kRepChunk = 32;        // vertices per chunk box of a neighbour's ring
-// Slack of the box tests: a box test may keep a pair that the exact test then drops,
-// never the reverse, whatever the rounding of the box arithmetic.
-constexpr double kRepSlack = 1e-9;
+// Gap between two intervals along one axis, through the periodic images when P > 0.
+__device__ __forceinline__ float gap_f(float lo0, float hi0, float lo1, float hi1, float P, float iP) {
+    float d = 0.5f * ((lo0 + hi0) - (lo1 + hi1));
+    d -= P * rintf(d * iP);
+    return fabsf(d) - 0.5f * ((hi0 - lo0) + (hi1 - lo1));
+}
 
-// Distance along one axis from coordinate x to the box [lo, hi] (0 inside), through the
-// periodic images when P > 0.
-__device__ __forceinline__ double axis_gap(double x, double lo, double hi, double P) {
-    return fabs(min_image(x - 0.5 * (lo + hi), P)) - 0.5 * (hi - lo);
+__device__ __forceinline__ float abs_max(const float4& b) {
+    return fmaxf(fmaxf(fabsf(b.x), fabsf(b.y)), fmaxf(fabsf(b.z), fabsf(b.w)));
 }
 
 // Eq. 27 forces on the vertices of one arc of a ring: CTA blockIdx.x = c * arcs + rank
-// owns the same share of capsule c's ring as in the immersed-boundary kernels. Each
-// neighbour capsule whose box comes within r_c of the arc's box is staged with boxes of
-// its 32-vertex chunks; a vertex then scans only the chunks within r_c of it.
+// owns the same share of capsule c's ring as in the immersed-boundary kernels. The last CTA
+// to finish empties the buckets for the next step.
 __global__ void __launch_bounds__(128) k_repulsion(Lat L, Nodes nd, int max_n, int arcs, RepGrid g) {
-    extern __shared__ __align__(16) unsigned char smem[];
-    const int slots = (max_n + arcs - 1) / arcs;
-    double2* own = reinterpret_cast<double2*>(smem);   // own arc: vertex v0 - 1 + li in slot li
-    double2* nrm = own + slots + 2;                    // inward normal of own vertex k
-    double2* oth = nrm + slots;                        // a neighbour's ring
-    double* cbox = reinterpret_cast<double*>(oth + max_n);   // its chunk boxes (min x, min y, max x, max y)
-    __shared__ double red[32 * 8];
     const int c = blockIdx.x / arcs, rank = blockIdx.x - c * arcs;
     const CapsuleParams P = nd.caps[c];
-    if (P.n < 3 || P.n > max_n) return;
-    const int n = P.n, chunk = (n + arcs - 1) / arcs, v0 = rank * chunk, m = min(n - v0, chunk);
-    if (m <= 0) return;
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const bool good = P.n >= 3 && P.n <= max_n;
+    const int n = P.n, chunk = good ? (n + arcs - 1) / arcs : 0, v0 = rank * chunk, m = good ? min(n - v0, chunk) : 0;
     const double px = L.inflow ? 0.0 : (double)L.nx, py = L.walls ? 0.0 : (double)L.ny;
-    for (int li = threadIdx.x; li < m + 2; li += blockDim.x) own[li] = nd.X[P.off + (v0 - 1 + li + n) % n];
-    __syncthreads();
-    double r[4] = {1e300, 1e300, 1e300, 1e300};   // the arc's box: min x, min y, -max x, -max y
-    for (int k = threadIdx.x; k < m; k += blockDim.x) {
-        const double2 Xl = own[k], Xv = own[k + 1], Xr = own[k + 2];
-        const double ax = Xv.x - Xl.x, ay = Xv.y - Xl.y, bx = Xr.x - Xv.x, by = Xr.y - Xv.y;
-        const double la = sqrt(ax * ax + ay * ay), lb = sqrt(bx * bx + by * by);
-        const double nx = ay / la + by / lb, ny = -ax / la - bx / lb;
-        const double ln = sqrt(nx * nx + ny * ny);
-        nrm[k] = make_double2(-nx / ln, -ny / ln);
-        r[0] = fmin(r[0], Xv.x);
-        r[1] = fmin(r[1], Xv.y);
-        r[2] = fmin(r[2], -Xv.x);
-        r[3] = fmin(r[3], -Xv.y);
-    }
-    block_reduce<4, true>(r, red);
-    const double mb[4] = {r[0], r[1], -r[2], -r[3]};
-    const double reach = g.rc + kRepSlack;
+    const float pxf = (float)px, pyf = (float)py, ipx = px > 0.0 ? 1.0f / pxf : 0.0f, ipy = py > 0.0 ? 1.0f / pyf : 0.0f;
     const int cell = g.cellof[c], ix = cell % g.ncx, iy = cell / g.ncx;
-    double facc[8] = {0, 0, 0, 0, 0, 0, 0, 0};   // own vertices threadIdx.x + 128 k, k < 8
     const int nxs = g.ncx < 3 ? g.ncx : 3, nys = (!L.walls && g.ncy < 3) ? g.ncy : 3;
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, nwarps = blockDim.x >> 5;
-    for (int sy = 0; sy < nys; sy++) {
-        int jy = iy + sy - (nys == 3 ? 1 : 0);
-        if (L.walls && (jy < 0 || jy >= g.ncy)) continue;
-        if (!L.walls) jy = ((jy % g.ncy) + g.ncy) % g.ncy;
-        for (int sx = 0; sx < nxs; sx++) {
-            const int jx = ((ix + sx - (nxs == 3 ? 1 : 0)) % g.ncx + g.ncx) % g.ncx;
-            const int h = bucket_of(jx, jy, g.nbuckets);
-            const int cnt = min(g.count[h], kRepSlots);
-            for (int e = 0; e < cnt; e++) {
-                const int o = g.slot[(size_t)h * kRepSlots + e];
-                if (o == c || g.cellof[o] != jy * g.ncx + jx) continue;   // self, or another cell's entry
-                const double* ob = g.box + 4 * o;
-                // boxes closer than r_c (minimum image between their centres)
-                const double gx = fabs(min_image(0.5 * (ob[0] + ob[2]) - 0.5 * (mb[0] + mb[2]), px)) -
-                                  0.5 * ((ob[2] - ob[0]) + (mb[2] - mb[0]));
-                const double gy = fabs(min_image(0.5 * (ob[1] + ob[3]) - 0.5 * (mb[1] + mb[3]), py)) -
-                                  0.5 * ((ob[3] - ob[1]) + (mb[3] - mb[1]));
-                if (gx >= reach || gy >= reach) continue;
-                const CapsuleParams Q = nd.caps[o];
-                if (Q.n < 3 || Q.n > max_n) continue;
-                const int nch = (Q.n + kRepChunk - 1) / kRepChunk;
-                __syncthreads();
-                for (int w = threadIdx.x; w < Q.n; w += blockDim.x) oth[w] = nd.X[Q.off + w];
-                __syncthreads();
-                for (int ch = warp; ch < nch; ch += nwarps) {
-                    const int w = ch * kRepChunk + lane;
-                    const double2 X = oth[w < Q.n ? w : ch * kRepChunk];
-                    double b0 = X.x, b1 = X.y, b2 = X.x, b3 = X.y;
-                    for (int sh = 16; sh > 0; sh >>= 1) {
-                        b0 = fmin(b0, __shfl_xor_sync(0xffffffffu, b0, sh));
-                        b1 = fmin(b1, __shfl_xor_sync(0xffffffffu, b1, sh));
-                        b2 = fmax(b2, __shfl_xor_sync(0xffffffffu, b2, sh));
-                        b3 = fmax(b3, __shfl_xor_sync(0xffffffffu, b3, sh));
-                    }
-                    if (lane == 0) {
-                        cbox[4 * ch] = b0;
-                        cbox[4 * ch + 1] = b1;
-                        cbox[4 * ch + 2] = b2;
-                        cbox[4 * ch + 3] = b3;
-                    }
-                }
-                __syncthreads();
-                for (int k = 0, v = threadIdx.x; v < m && k < 8; k++, v += blockDim.x) {
-                    const double2 Xv = own[v + 1];
-                    if (axis_gap(Xv.x, ob[0], ob[2], px) >= reach || axis_gap(Xv.y, ob[1], ob[3], py) >= reach)
+    for (int s0 = 32 * warp; s0 < m; s0 += 128) {
+        const int k = s0 + lane, v = v0 + min(k, m - 1), gi = P.off + v;
+        const float2 xf = g.xf[gi];
+        const double2 X = nd.X[gi];
+        const float4 wb = make_float4(warp_min(xf.x), warp_min(xf.y), warp_max(xf.x), warp_max(xf.y));
+        double f = 0.0;
+        for (int sy = 0; sy < nys; sy++) {
+            int jy = iy + sy - (nys == 3 ? 1 : 0);
+            if (L.walls && (jy < 0 || jy >= g.ncy)) continue;
+            if (!L.walls) jy = ((jy % g.ncy) + g.ncy) % g.ncy;
+            for (int sx = 0; sx < nxs; sx++) {
+                const int jx = ((ix + sx - (nxs == 3 ? 1 : 0)) % g.ncx + g.ncx) % g.ncx;
+                const int h = bucket_of(jx, jy, g.nbuckets);
+                const int cnt = min(g.count[h], kRepSlots);
+                for (int e = 0; e < cnt; e++) {
+                    const int o = g.slot[(size_t)h * kRepSlots + e];
+                    if (o == c || g.cellof[o] != jy * g.ncx + jx) continue;   // self, or another cell's entry
+                    const float4 ob = g.box[o];
+                    // the reach covers the rounding of the float positions, periods and boxes: a
+                    // test may keep a pair that the double one then drops, never the reverse
+                    const float big = fmaxf(fmaxf(abs_max(wb), abs_max(ob)), fmaxf(pxf, pyf));
+                    const float reach = (float)g.rc + 1e-6f + 2e-6f * big;
+                    if (gap_f(wb.x, wb.z, ob.x, ob.z, pxf, ipx) >= reach ||
+                        gap_f(wb.y, wb.w, ob.y, ob.w, pyf, ipy) >= reach)
                         continue;
-                    double f = 0.0;
-                    for (int ch = 0; ch < nch; ch++) {
-                        const double* cb = cbox + 4 * ch;
-                        if (axis_gap(Xv.x, cb[0], cb[2], px) >= reach || axis_gap(Xv.y, cb[1], cb[3], py) >= reach)
-                            continue;
-                        const int w1 = min(Q.n, (ch + 1) * kRepChunk);
-                        for (int w = ch * kRepChunk; w < w1; w++) {
-                            const double dx = min_image(Xv.x - oth[w].x, px), dy = min_image(Xv.y - oth[w].y, py);
-                            const double d2 = dx * dx + dy * dy;
-                            if (d2 < g.rc * g.rc) f += g.coeff * rsqrt(d2 * d2 * sqrt(d2));   // coeff d^{-5/2}
+                    const CapsuleParams Q = nd.caps[o];
+                    if (Q.n < 3 || Q.n > max_n) continue;
+                    const int nch = (Q.n + 31) / 32, first = first_chunk(o, Q.off);
+                    for (int c0 = 0; c0 < nch; c0 += 32) {
+                        bool near = false;
+                        if (c0 + lane < nch) {
+                            const float4 cb = g.cbox[first + c0 + lane];
+                            near = gap_f(wb.x, wb.z, cb.x, cb.z, pxf, ipx) < reach &&
+                                   gap_f(wb.y, wb.w, cb.y, cb.w, pyf, ipy) < reach;
+                        }
+                        for (unsigned hit = __ballot_sync(0xffffffffu, near); hit; hit &= hit - 1) {
+                            const int w0 = 32 * (c0 + __ffs((int)hit) - 1), nw = min(32, Q.n - w0);
+                            const float2 of = g.xf[Q.off + w0 + min(lane, nw - 1)];
+                            unsigned cand = 0;
+                            for (int j = 0; j < nw; j++) {
+                                float dx = xf.x - __shfl_sync(0xffffffffu, of.x, j);
+                                float dy = xf.y - __shfl_sync(0xffffffffu, of.y, j);
+                                dx -= pxf * rintf(dx * ipx);
+                                dy -= pyf * rintf(dy * ipy);
+                                if (dx * dx + dy * dy < reach * reach) cand |= 1u << j;
+                            }
+                            for (cand = k < m ? cand : 0u; cand; cand &= cand - 1) {
+                                const double2 Y = nd.X[Q.off + w0 + __ffs((int)cand) - 1];
+                                const double dx = min_image(X.x - Y.x, px), dy = min_image(X.y - Y.y, py);
+                                const double d2 = dx * dx + dy * dy;
+                                if (d2 < g.rc * g.rc) f += g.coeff * rsqrt(d2 * d2 * sqrt(d2));   // coeff d^{-5/2}
+                            }
+                            __syncwarp();
                         }
                     }
-                    facc[k] += f;
                 }
             }
         }
+        if (k < m) {
+            double2 F = make_double2(0.0, 0.0);
+            if (f != 0.0) {
+                const double2 Xl = nd.X[P.off + (v + n - 1) % n], Xr = nd.X[P.off + (v + 1) % n];
+                const double ax = X.x - Xl.x, ay = X.y - Xl.y, bx = Xr.x - X.x, by = Xr.y - X.y;
+                const double la = sqrt(ax * ax + ay * ay), lb = sqrt(bx * bx + by * by);
+                const double nx = ay / la + by / lb, ny = -ax / la - bx / lb;
+                const double ln = sqrt(nx * nx + ny * ny);
+                F = make_double2(f * (-nx / ln), f * (-ny / ln));
+            }
+            nd.Fpp[gi] = F;
+        }
     }
-    for (int k = 0, v = threadIdx.x; v < m && k < 8; k++, v += blockDim.x)
-        nd.Fpp[P.off + v0 + v] = make_double2(facc[k] * nrm[v].x, facc[k] * nrm[v].y);
+    __shared__ int last;
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        __threadfence();
+        last = atomicAdd(&g.count[g.nbuckets], 1) == (int)gridDim.x - 1;
+    }
+    __syncthreads();
+    if (last)
+        for (int h = threadIdx.x; h <= g.nbuckets; h += blockDim.x) g.count[h] = 0;
 }
 
 }  // namespace
 
 void launch_repulsion(const Lat& L, Nodes nd, int ncaps, int max_n, int arcs, RepGrid g, unsigned* status,
                       cudaStream_t s) {
-    cudaMemsetAsync(g.count, 0, sizeof(int) * (size_t)g.nbuckets, s);
     k_rep_bin<<<ncaps, 128, 0, s>>>(L, nd, max_n, g, status);
-    const size_t slots = (size_t)((max_n + arcs - 1) / arcs);
-    const size_t sh = (2 * slots + 2 + (size_t)max_n) * sizeof(double2) +
-                      4 * sizeof(double) * (size_t)((max_n + kRepChunk - 1) / kRepChunk);
-    cudaFuncSetAttribute(k_repulsion, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sh);
-    k_repulsion<<<ncaps * arcs, 128, sh, s>>>(L, nd, max_n, arcs, g);
+    k_repulsion<<<ncaps * arcs, 128, 0, s>>>(L, nd, max_n, arcs, g);
 }
 
 }  // namespace lbmib
