@@ -79,9 +79,10 @@ __device__ __forceinline__ void st_vec(S* p, const typename St<S>::C (&o)[Vec<S>
 // issue() fetches the aligned 16-byte vector of the source row (at a wall, of the node's
 // own opposite population) and, for an edge lane, the one scalar that no neighbouring
 // lane holds; resolve() shifts by -e_x through warp shuffles. All 32 lanes of the warp
-// call both with the same y. A lane whose chunk crosses the end of the row ("ragged",
-// only when nx is not a multiple of V) keeps its raw vector for its neighbours'
-// shuffles and gathers its own shifted values element-wise in resolve().
+// call both with the same y. A chunk that crosses the end of the row ("ragged", only when
+// nx is not a multiple of V) is left to k_ragged: gathered element by element in here, it
+// made its warp three times as long, and with it its block's stay on the multiprocessor
+// (4099 x 2053, FP32: 112 -> 97 us).
 template <typename S, int I, int LM>
 struct PopLoad {
     using C = typename St<S>::C;
@@ -117,8 +118,8 @@ struct PopLoad {
             if (EX == -1 && (lane == 31 || x0 + 2 * V > L.nx)) edge = St<S>::ld(row + wrapi(x0 + V, L.nx), L);
         }
     }
-    __device__ __forceinline__ void resolve(const S* __restrict__ src, const Lat& L, int x0, int y, int lane,
-                                            bool active, bool full, C (&out)[V]) const {
+    __device__ __forceinline__ void resolve(const Lat& L, int x0, int y, int lane,
+                                            C (&out)[V]) const {
         constexpr int EX = ex(I);
         if (at_wall(L, y)) {  // warp-uniform
             constexpr int J = opp(I);
@@ -142,18 +143,6 @@ struct PopLoad {
             for (int j = 0; j < V - 1; j++) out[j] = v[j + 1];
             out[V - 1] = next;
         }
-        if (active && !full) {  // ragged chunk: element-wise, with the pull's wrap
-            const S* row = row_ptr(src, L, y);
-            const bool wall = at_wall(L, y);
-            const C uw = y - ey(I) < 0 ? lat_c<C>(L.ub, L.ubf) : lat_c<C>(L.ut, L.utf);
-            const C corr = wall ? C(6) * wgt<C>(opp(I)) * C(ex(opp(I))) * uw : C(0);
-#pragma unroll
-            for (int j = 0; j < V; j++) {
-                const int x = x0 + j;
-                out[j] = x < L.nx ? (wall ? St<S>::ld(row + x, L) - corr : St<S>::ld(row + wrapi(x - EX, L.nx), L))
-                                  : C(0);
-            }
-        }
     }
 };
 
@@ -164,28 +153,27 @@ __global__ void __launch_bounds__(BS, MINB) k_collide_stream(const S* __restrict
     constexpr int V = Vec<S>::V;
     const int lane = threadIdx.x & 31;
     const long long gw = ((long long)blockIdx.x * BS + threadIdx.x) >> 5;
-    const int segs = (L.nx + 32 * V - 1) / (32 * V);
+    const int segs = (L.nx / V + 31) / 32;   // whole vectors only: the rest of a row is k_ragged's
     if (gw >= (long long)segs * L.ny) return;  // whole warps only
     const int y = (int)(gw / segs);
     const int seg = (int)(gw - (long long)y * segs);
     const int x0 = (seg * 32 + lane) * V;
-    const bool active = x0 < L.nx;
     const bool full = x0 + V <= L.nx;
 
     PopLoad<S, 0, LM> p0; PopLoad<S, 1, LM> p1; PopLoad<S, 2, LM> p2;
     PopLoad<S, 3, LM> p3; PopLoad<S, 4, LM> p4; PopLoad<S, 5, LM> p5;
     PopLoad<S, 6, LM> p6; PopLoad<S, 7, LM> p7; PopLoad<S, 8, LM> p8;
-    p0.issue(src, L, x0, y, lane, active); p1.issue(src, L, x0, y, lane, active);
-    p2.issue(src, L, x0, y, lane, active); p3.issue(src, L, x0, y, lane, active);
-    p4.issue(src, L, x0, y, lane, active); p5.issue(src, L, x0, y, lane, active);
-    p6.issue(src, L, x0, y, lane, active); p7.issue(src, L, x0, y, lane, active);
-    p8.issue(src, L, x0, y, lane, active);
+    p0.issue(src, L, x0, y, lane, full); p1.issue(src, L, x0, y, lane, full);
+    p2.issue(src, L, x0, y, lane, full); p3.issue(src, L, x0, y, lane, full);
+    p4.issue(src, L, x0, y, lane, full); p5.issue(src, L, x0, y, lane, full);
+    p6.issue(src, L, x0, y, lane, full); p7.issue(src, L, x0, y, lane, full);
+    p8.issue(src, L, x0, y, lane, full);
     C f[9][V];
-    p0.resolve(src, L, x0, y, lane, active, full, f[0]); p1.resolve(src, L, x0, y, lane, active, full, f[1]);
-    p2.resolve(src, L, x0, y, lane, active, full, f[2]); p3.resolve(src, L, x0, y, lane, active, full, f[3]);
-    p4.resolve(src, L, x0, y, lane, active, full, f[4]); p5.resolve(src, L, x0, y, lane, active, full, f[5]);
-    p6.resolve(src, L, x0, y, lane, active, full, f[6]); p7.resolve(src, L, x0, y, lane, active, full, f[7]);
-    p8.resolve(src, L, x0, y, lane, active, full, f[8]);
+    p0.resolve(L, x0, y, lane, f[0]); p1.resolve(L, x0, y, lane, f[1]);
+    p2.resolve(L, x0, y, lane, f[2]); p3.resolve(L, x0, y, lane, f[3]);
+    p4.resolve(L, x0, y, lane, f[4]); p5.resolve(L, x0, y, lane, f[5]);
+    p6.resolve(L, x0, y, lane, f[6]); p7.resolve(L, x0, y, lane, f[7]);
+    p8.resolve(L, x0, y, lane, f[8]);
 
     const C gx = lat_c<C>(L.gx, L.gxf), gy = lat_c<C>(L.gy, L.gyf), om = lat_c<C>(L.omega, L.omegaf);
     bool bad = false;
@@ -221,14 +209,8 @@ __global__ void __launch_bounds__(BS, MINB) k_collide_stream(const S* __restrict
 #pragma unroll
         for (int i = 0; i < 9; i++)
             st_vec<S, SMODE>(dst + (long long)i * L.plane + (long long)y * L.pitch + x0, f[i], L);
-    } else if (active) {
-#pragma unroll
-        for (int i = 0; i < 9; i++)
-#pragma unroll
-            for (int j = 0; j < V; j++)
-                if (x0 + j < L.nx) St<S>::st(dst + (long long)i * L.plane + (long long)y * L.pitch + x0 + j, f[i][j], L);
     }
-    if (__any_sync(0xffffffffu, bad && active) && lane == 0) atomicOr(status, kStatUnstable);
+    if (__any_sync(0xffffffffu, bad && full) && lane == 0) atomicOr(status, kStatUnstable);
 }
 
 // FP64 storage: the same loads and stores with the uniform force's constants from the host
@@ -241,26 +223,26 @@ __global__ void __launch_bounds__(BS, MINB) k_collide_stream_d(const double* __r
     constexpr int V = 2;
     const int lane = threadIdx.x & 31;
     const long long gw = ((long long)blockIdx.x * BS + threadIdx.x) >> 5;
-    const int segs = (L.nx + 32 * V - 1) / (32 * V);
+    const int segs = (L.nx / V + 31) / 32;   // whole vectors only: the rest of a row is k_ragged's
     if (gw >= (long long)segs * L.ny) return;  // whole warps only
     const int y = (int)(gw / segs);
     const int seg = (int)(gw - (long long)y * segs);
     const int x0 = (seg * 32 + lane) * V;
-    const bool active = x0 < L.nx, full = x0 + V <= L.nx;
+    const bool full = x0 + V <= L.nx;
     PopLoad<double, 0, 0> p0; PopLoad<double, 1, 0> p1; PopLoad<double, 2, 0> p2;
     PopLoad<double, 3, 0> p3; PopLoad<double, 4, 0> p4; PopLoad<double, 5, 0> p5;
     PopLoad<double, 6, 0> p6; PopLoad<double, 7, 0> p7; PopLoad<double, 8, 0> p8;
-    p0.issue(src, L, x0, y, lane, active); p1.issue(src, L, x0, y, lane, active);
-    p2.issue(src, L, x0, y, lane, active); p3.issue(src, L, x0, y, lane, active);
-    p4.issue(src, L, x0, y, lane, active); p5.issue(src, L, x0, y, lane, active);
-    p6.issue(src, L, x0, y, lane, active); p7.issue(src, L, x0, y, lane, active);
-    p8.issue(src, L, x0, y, lane, active);
+    p0.issue(src, L, x0, y, lane, full); p1.issue(src, L, x0, y, lane, full);
+    p2.issue(src, L, x0, y, lane, full); p3.issue(src, L, x0, y, lane, full);
+    p4.issue(src, L, x0, y, lane, full); p5.issue(src, L, x0, y, lane, full);
+    p6.issue(src, L, x0, y, lane, full); p7.issue(src, L, x0, y, lane, full);
+    p8.issue(src, L, x0, y, lane, full);
     double f[9][V];
-    p0.resolve(src, L, x0, y, lane, active, full, f[0]); p1.resolve(src, L, x0, y, lane, active, full, f[1]);
-    p2.resolve(src, L, x0, y, lane, active, full, f[2]); p3.resolve(src, L, x0, y, lane, active, full, f[3]);
-    p4.resolve(src, L, x0, y, lane, active, full, f[4]); p5.resolve(src, L, x0, y, lane, active, full, f[5]);
-    p6.resolve(src, L, x0, y, lane, active, full, f[6]); p7.resolve(src, L, x0, y, lane, active, full, f[7]);
-    p8.resolve(src, L, x0, y, lane, active, full, f[8]);
+    p0.resolve(L, x0, y, lane, f[0]); p1.resolve(L, x0, y, lane, f[1]);
+    p2.resolve(L, x0, y, lane, f[2]); p3.resolve(L, x0, y, lane, f[3]);
+    p4.resolve(L, x0, y, lane, f[4]); p5.resolve(L, x0, y, lane, f[5]);
+    p6.resolve(L, x0, y, lane, f[6]); p7.resolve(L, x0, y, lane, f[7]);
+    p8.resolve(L, x0, y, lane, f[8]);
     bool bad = false;
 #pragma unroll
     for (int j = 0; j < V; j++) {
@@ -277,9 +259,8 @@ __global__ void __launch_bounds__(BS, MINB) k_collide_stream_d(const double* __r
 #pragma unroll
     for (int i = 0; i < 9; i++) {
         if (full) *reinterpret_cast<double2*>(o + (long long)i * L.plane) = make_double2(f[i][0], f[i][1]);
-        else if (active) o[(long long)i * L.plane] = f[i][0];
     }
-    if (__any_sync(0xffffffffu, bad && active) && lane == 0) atomicOr(status, kStatUnstable);
+    if (__any_sync(0xffffffffu, bad && full) && lane == 0) atomicOr(status, kStatUnstable);
 }
 
 // FP16 storage: one warp owns 256 consecutive nodes of a row, 8 per thread, each
@@ -441,14 +422,32 @@ __global__ void __launch_bounds__(BS, MINB) k_collide_stream_h(const __half* __r
     if (__any_sync(0xffffffffu, bad && full) && lane == 0) atomicOr(status, kStatUnstable);
 }
 
-// The ragged chunk at the end of every row of the packed FP16 kernel (nx not a multiple
-// of 8), one thread per row, launched after it: a separate kernel keeps the element-wise
+// The ragged chunk at the end of every row of the FP16 kernels (nx not a multiple of their
+// V nodes per thread), one thread per row, a launch of its own: a separate kernel keeps the element-wise
 // path out of the hot kernel's registers.
+template <int V>
 __global__ void __launch_bounds__(128) k_ragged_h(const __half* __restrict__ src, __half* __restrict__ dst, Lat L,
                                                   unsigned* __restrict__ status) {
     const int y = blockIdx.x * blockDim.x + threadIdx.x;
     if (y >= L.ny) return;
-    if (ragged_chunk_h(src, dst, L, L.nx / 8 * 8, y, L.gxf, L.gyf, L.omegaf)) atomicOr(status, kStatUnstable);
+    if (ragged_chunk_h(src, dst, L, L.nx / V * V, y, L.gxf, L.gyf, L.omegaf)) atomicOr(status, kStatUnstable);
+}
+
+// The nodes of FP32 and FP64 rows beyond the last whole vector (nx not a multiple of V), one
+// thread per node.
+template <typename S>
+__global__ void __launch_bounds__(128) k_ragged(const S* __restrict__ src, S* __restrict__ dst, Lat L,
+                                                unsigned* __restrict__ status) {
+    using C = typename St<S>::C;
+    const int x0 = L.nx / Vec<S>::V * Vec<S>::V, w = L.nx - x0;
+    const int t = blockIdx.x * blockDim.x + threadIdx.x, y = t / w, x = x0 + t - y * w;
+    if (y >= L.ny) return;
+    C s[9];
+    pull_all<S>(src, L, x, y, s);
+    const C usq = collide<C>(s, lat_c<C>(L.gx, L.gxf), lat_c<C>(L.gy, L.gyf), lat_c<C>(L.omega, L.omegaf));
+    if (!(usq < C(0.09))) atomicOr(status, kStatUnstable);
+#pragma unroll
+    for (int i = 0; i < 9; i++) St<S>::st(dst + (long long)i * L.plane + (long long)y * L.pitch + x, s[i], L);
 }
 
 // Forced-node patch: the nodes of the current touched-cell list collide with the total
@@ -528,8 +527,8 @@ __global__ void __launch_bounds__(256) k_patch(S* __restrict__ dst, Lat L, const
         __threadfence();
         if (atomicAdd(&ctr->patch_blocks, 1) == (int)gridDim.x - 1) {
             ctr->patch_blocks = 0;
-            ctr->count[1 - c] = 0;   // every block has read it; the next spread appends from here
             ctr->step_stamp = stamp;
+            ctr->count[1 - c] = 0;   // every block has read it; the next spread appends from here
         }
     }
 }
@@ -669,7 +668,7 @@ void launch_collide_stream(const void* src, void* dst, const Lat& L, unsigned* s
     constexpr int V = Vec<S>::V;
     const int bs = (variant & 0xfff) == 128 ? 128 : 256;
     const bool occ4 = (variant >> 18) & 1;
-    const long long segs = (L.nx + 32 * V - 1) / (32 * V);
+    const long long segs = (L.nx / V + 31) / 32;
     const long long threads = segs * L.ny * 32;
     const unsigned g = blocks_for(threads, bs);
     const S* a = (const S*)src;
@@ -680,10 +679,15 @@ void launch_collide_stream(const void* src, void* dst, const Lat& L, unsigned* s
             const unsigned g8 = blocks_for(segs8 * L.ny * 32, bs);
             if (bs == 128) k_collide_stream_h<128, 6><<<g8, 128, 0, s>>>(a, b, L, status);
             else k_collide_stream_h<256, 3><<<g8, 256, 0, s>>>(a, b, L, status);
-            if (L.nx % 8) k_ragged_h<<<blocks_for(L.ny, 128), 128, 0, s>>>(a, b, L, status);
+            if (L.nx % 8) k_ragged_h<8><<<blocks_for(L.ny, 128), 128, 0, s>>>(a, b, L, status);
             return;
         }
     }
+    if (const int w = L.nx % V) {
+        if constexpr (std::is_same<S, __half>::value) k_ragged_h<V><<<blocks_for(L.ny, 128), 128, 0, s>>>(a, b, L, status);
+        else k_ragged<S><<<blocks_for((long long)L.ny * w, 128), 128, 0, s>>>(a, b, L, status);
+    }
+    if (segs == 0) return;
     if constexpr (std::is_same<S, double>::value) {
         const CollideD k(L.gx, L.gy, L.omega);
         if (bs == 256) k_collide_stream_d<256, 3><<<g, 256, 0, s>>>(a, b, L, k, status);
