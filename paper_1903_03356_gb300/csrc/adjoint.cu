@@ -41,6 +41,8 @@
 namespace lbmib {
 namespace {
 
+using lbmib::operator-;   // of double2, beside the scalar types' below
+
 // ---------------------------------------------------------------------------------
 // Dual numbers: a value and its derivative along one direction.
 // ---------------------------------------------------------------------------------
@@ -58,7 +60,6 @@ __device__ __forceinline__ Dual operator/(Dual a, Dual b) {
 }
 __device__ __forceinline__ Dual operator*(double s, Dual a) { return {s * a.v, s * a.d}; }
 __device__ __forceinline__ Dual operator+(Dual a, double s) { return {a.v + s, a.d}; }
-__device__ __forceinline__ Dual operator-(double s, Dual a) { return {s - a.v, -a.d}; }
 __device__ __forceinline__ Dual dsqrt(Dual a) {
     const double r = sqrt(a.v);
     return {r, a.d / (2.0 * r)};
@@ -230,47 +231,6 @@ __device__ Shape shape_with_derivatives(const Lat& L, double X, double Y) {
 
 __device__ __forceinline__ int support_cell(const Lat& L, const Shape& s, int a, int b) {
     return support_row(L, s.cy + b - 1) * L.nx + wrapi(s.cx + a - 1, L.nx);
-}
-
-// ---------------------------------------------------------------------------------
-// Membrane force of vertex v with unit constants, split into its stretch (Eq. 11),
-// bending (Eq. 13) and area (Eq. 14) parts: F_v = k_s Fs + k_b Fb + k_a Fa. Written
-// for any scalar type so that dual numbers give its directional derivative.
-// ---------------------------------------------------------------------------------
-template <typename T, typename GetX>
-__device__ void membrane_parts(int v, int n, GetX X, const double* L0, const double* c0, const double* s0, T A,
-                               double A0, P2<T>& Fs, P2<T>& Fb, P2<T>& Fa) {
-    auto idx = [n](int k) { return k < 0 ? k + n : (k >= n ? k - n : k); };
-    P2<T> p[5];   // X_{v-2} .. X_{v+2}
-#pragma unroll
-    for (int j = 0; j < 5; j++) p[j] = X(idx(v + j - 2));
-    // stretch: elements v-1 (p1 -> p2) and v (p2 -> p3)
-    {
-        const P2<T> bl = p[2] - p[1], br = p[3] - p[2];
-        const T ll = dsqrt(bl.x * bl.x + bl.y * bl.y), lr = dsqrt(br.x * br.x + br.y * br.y);
-        const T tl = -((ll + (-L0[idx(v - 1)])) / ll), tr = -((lr + (-L0[v])) / lr);
-        Fs.x = tr * (p[2].x - p[3].x) + tl * (p[2].x - p[1].x);
-        Fs.y = tr * (p[2].y - p[3].y) + tl * (p[2].y - p[1].y);
-    }
-    // bending: angles at v-1, v, v+1 (centres p[1], p[2], p[3])
-    T bs[3];
-    P2<T> bdl[3], bdr[3];
-#pragma unroll
-    for (int j = 0; j < 3; j++) {
-        const P2<T> a = p[j + 1] - p[j], b = p[j + 2] - p[j + 1];
-        const T a2 = a.x * a.x + a.y * a.y, b2 = b.x * b.x + b.y * b.y;
-        const T cr = a.x * b.y - a.y * b.x, dt = a.x * b.x + a.y * b.y;
-        const int k = idx(v + j - 1);
-        bs[j] = (c0[k] * cr - s0[k] * dt) / dsqrt(a2 * b2);
-        bdl[j] = {(-a.y) / a2, a.x / a2};
-        bdr[j] = {(-b.y) / b2, b.x / b2};
-    }
-    Fb.x = bs[1] * (bdl[1].x + bdr[1].x) - bs[2] * bdl[2].x - bs[0] * bdr[0].x;
-    Fb.y = bs[1] * (bdl[1].y + bdr[1].y) - bs[2] * bdl[2].y - bs[0] * bdr[0].y;
-    // area: (1 - A / A0) / 6 * (dr.y + dl.y, -(dr.x + dl.x)), dr + dl = X_{v+1} - X_{v-1}
-    const T fa = (1.0 / 6.0) * (1.0 - A / mk(A0));
-    Fa.x = fa * (p[3].y - p[1].y);
-    Fa.y = -(fa * (p[3].x - p[1].x));
 }
 
 // ---------------------------------------------------------------------------------
@@ -545,23 +505,24 @@ __global__ void __launch_bounds__(256) k_adj_lattice(const S* __restrict__ post0
             // adjoint, e_x -> e_x with force adjoint (1, 0). Those parts are split off in
             // double (weighted mean and first moments of p-bar) and only the remainder
             // goes through the float transpose.
-            double c0 = 0.0, ca = 0.0, cb = 0.0;
-#pragma unroll
-            for (int i = 0; i < 9; i++) {
-                const double w = wgt<double>(i);
-                c0 += w * pb[i];
-                ca += 3.0 * w * ex(i) * pb[i];
-                cb += 3.0 * w * ey(i) * pb[i];
-            }
+            // (By sums and differences of opposite directions: the kernel is bound by its FP64
+            // instructions, here 80 per node against 108 term by term: 21.9 -> 17 us on 512 x 128.)
+            const double p1 = pb[1] + pb[3], d1 = pb[1] - pb[3], p2 = pb[2] + pb[4], d2 = pb[2] - pb[4];
+            const double p5 = pb[5] + pb[7], d5 = pb[5] - pb[7], p6 = pb[6] + pb[8], d6 = pb[6] - pb[8];
+            const double c0 = fma(4.0 / 9.0, pb[0], fma(1.0 / 9.0, p1 + p2, (1.0 / 36.0) * (p5 + p6)));
+            const double ca = fma(1.0 / 3.0, d1, (1.0 / 12.0) * (d5 - d6));
+            const double cb = fma(1.0 / 3.0, d2, (1.0 / 12.0) * (d5 + d6));
+            const double xp = c0 + ca, xm = c0 - ca;
+            const double base[9] = {c0, xp, c0 + cb, xm, c0 - cb, xp + cb, xm + cb, xm - cb, xp - cb};
             float sf[9], rf[9], sbf[9], fx, fy;
 #pragma unroll
             for (int i = 0; i < 9; i++) {
                 sf[i] = (float)sc[i];
-                rf[i] = (float)(pb[i] - c0 - ca * ex(i) - cb * ey(i));
+                rf[i] = (float)(pb[i] - base[i]);
             }
             collide_adjoint<float>(sf, (float)Fx, (float)Fy, L.omegaf, rf, sbf, fx, fy);
 #pragma unroll
-            for (int i = 0; i < 9; i++) sb[i] = c0 + ca * ex(i) + cb * ey(i) + (double)sbf[i];
+            for (int i = 0; i < 9; i++) sb[i] = base[i] + (double)sbf[i];
             Fbx = ca + (double)fx;
             Fby = cb + (double)fy;
         }
@@ -599,35 +560,97 @@ __global__ void __launch_bounds__(256) k_adj_lattice(const S* __restrict__ post0
     }
 }
 
+// 1 / sqrt(x) in double: the hardware's approximation (about 22 bits) and two Newton steps.
+__device__ __forceinline__ double rsqrt_newton(double x) {
+    double y;
+    asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
+    y = fma(0.5 * y, fma(-x * y, y, 1.0), y);
+    return fma(0.5 * y, fma(-x * y, y, 1.0), y);
+}
+
+// Shared memory of the kernels that call membrane_transpose: the staged ring and three more
+// double2 per vertex.
+inline size_t transpose_smem(int max_n) {
+    return ring_smem_bytes(max_n) + 3 * (size_t)max_n * sizeof(double2);
+}
+
 // Membrane transpose of one capsule (collective): with the vertices in sm.X and F-bar in
 // sm.ext, adds d/de F_v(X + e F-bar) (= (dF/dX)^T F-bar, the Jacobian being symmetric)
 // to sm.xd[v], and F-bar . dF/dk to the k_s and k_b gradients of capsule `cap`.
+// One CTA per capsule is bound by its FP64 instructions (one per warp and 64 cycles), so the
+// forces are written over elements and angles, each formed once and differentiated by hand
+// (e' the derivative along F-bar, r = 1/|e|, s = e.e'):
+//   element: T = (1 - L0 r) e, T' = (1 - L0 r) e' + L0 r^3 s e,
+//            n = r^2 (-e_y, e_x), n' = r^2 (-e'_y, e'_x) - 2 r^2 s n
+//   angle:   g = sin(theta - theta_0) = (c0 a x b - s0 a.b) r_a r_b, g' likewise
+//   vertex:  F_s = T_v - T_{v-1},  F_b = (g_v - g_{v-1}) n_{v-1} + (g_v - g_{v+1}) n_v,
+// about 90 of them per vertex (as dual numbers over the five-vertex stencil some 650: the
+// Dynamic update transpose of one 128-vertex ring 23.9 -> 8 us).
 __device__ void membrane_transpose(const CapSmem& sm, const CapsuleParams& P, const Nodes& nd, int cap, int ncaps,
                                    double* grad) {
     const int n = P.n, off = P.off;
+    double2* T = sm.bdl;
+    double2* Td = sm.bdr;
+    double* R = sm.sst;
+    double* S = sm.bs;
+    double2* N = reinterpret_cast<double2*>(sm.tile);
+    double2* Nd = N + n;
+    double2* G = Nd + n;   // (g, g')
+    const double2 X0 = sm.X[0], t0 = sm.ext[0];
     double ar[2] = {0.0, 0.0};
-    auto getd = [&](int k) {
-        const double2 p = sm.X[k], t = sm.ext[k];
-        return P2<Dual>{mk(p.x, t.x), mk(p.y, t.y)};
-    };
     for (int v = threadIdx.x; v < n; v += blockDim.x) {
-        const P2<Dual> p0 = getd(0), a = getd(v) - p0, b = getd(v + 1 == n ? 0 : v + 1) - p0;
-        const Dual c2 = a.x * b.y - b.x * a.y;
-        ar[0] += c2.v;
-        ar[1] += c2.d;
+        const int w = v + 1 == n ? 0 : v + 1;
+        const double2 e = sm.X[w] - sm.X[v], ed = sm.ext[w] - sm.ext[v];
+        const double r = rsqrt_newton(fma(e.x, e.x, e.y * e.y)), s = fma(e.x, ed.x, e.y * ed.y), r2 = r * r;
+        const double lr = nd.L0[off + v] * r, f = 1.0 - lr, k = lr * r2 * s, m = -2.0 * r2 * s;
+        T[v] = make_double2(f * e.x, f * e.y);
+        Td[v] = make_double2(fma(f, ed.x, k * e.x), fma(f, ed.y, k * e.y));
+        const double2 q = make_double2(-r2 * e.y, r2 * e.x);
+        N[v] = q;
+        Nd[v] = make_double2(fma(-r2, ed.y, m * q.x), fma(r2, ed.x, m * q.y));
+        R[v] = r;
+        S[v] = s * r2;
+        if (P.ka != 0.0) {   // twice the enclosed area about X_0, and its derivative
+            const double2 p = sm.X[v] - X0, pd = sm.ext[v] - t0;
+            ar[0] += p.x * e.y - p.y * e.x;
+            ar[1] += pd.x * e.y - pd.y * e.x + p.x * ed.y - p.y * ed.x;
+        }
     }
-    block_reduce<2, false>(ar, sm.red);
-    const Dual A = mk(0.5 * ar[0], 0.5 * ar[1]);
+    block_reduce<2, false>(ar, sm.red);   // also orders the elements before the angles
+    for (int v = threadIdx.x; v < n; v += blockDim.x) {
+        const int u = v == 0 ? n - 1 : v - 1, w = v + 1 == n ? 0 : v + 1;
+        const double2 a = sm.X[v] - sm.X[u], b = sm.X[w] - sm.X[v];
+        const double2 ad = sm.ext[v] - sm.ext[u], bd = sm.ext[w] - sm.ext[v];
+        const double c0 = nd.c0[off + v], s0 = nd.s0[off + v], rr = R[u] * R[v];
+        const double cr = fma(a.x, b.y, -a.y * b.x), dt = fma(a.x, b.x, a.y * b.y);
+        const double crd = fma(ad.x, b.y, -ad.y * b.x) + fma(a.x, bd.y, -a.y * bd.x);
+        const double dtd = fma(ad.x, b.x, ad.y * b.y) + fma(a.x, bd.x, a.y * bd.y);
+        const double g = fma(c0, cr, -s0 * dt) * rr;
+        G[v] = make_double2(g, fma(fma(c0, crd, -s0 * dtd), rr, -g * (S[u] + S[v])));
+    }
+    __syncthreads();
+    const double fa = P.ka != 0.0 ? (1.0 - 0.5 * ar[0] / P.A0) / 6.0 : 0.0;
+    const double fad = P.ka != 0.0 ? -0.5 * ar[1] / (6.0 * P.A0) : 0.0;
     double kk[2] = {0.0, 0.0};
     for (int v = threadIdx.x; v < n; v += blockDim.x) {
-        P2<Dual> Fs, Fb, Fa;
-        membrane_parts<Dual>(v, n, getd, nd.L0 + off, nd.c0 + off, nd.s0 + off, A, P.A0, Fs, Fb, Fa);
-        const double2 fb = sm.ext[v];
-        kk[0] += fb.x * Fs.x.v + fb.y * Fs.y.v;
-        kk[1] += fb.x * Fb.x.v + fb.y * Fb.y.v;
-        const double2 c = sm.xd[v];
-        sm.xd[v] = make_double2(c.x + P.ks * Fs.x.d + P.kb * Fb.x.d + P.ka * Fa.x.d,
-                                c.y + P.ks * Fs.y.d + P.kb * Fb.y.d + P.ka * Fa.y.d);
+        const int u = v == 0 ? n - 1 : v - 1, w = v + 1 == n ? 0 : v + 1;
+        const double2 fb = sm.ext[v], Fs = T[v] - T[u], Fsd = Td[v] - Td[u];
+        const double2 gu = G[u], gv = G[v], gw = G[w], nu = N[u], nv = N[v], nud = Nd[u], nvd = Nd[v];
+        const double hu = gv.x - gu.x, hw = gv.x - gw.x, hud = gv.y - gu.y, hwd = gv.y - gw.y;
+        const double2 Fb = make_double2(fma(hu, nu.x, hw * nv.x), fma(hu, nu.y, hw * nv.y));
+        const double2 Fbd = make_double2(fma(hud, nu.x, hu * nud.x) + fma(hwd, nv.x, hw * nvd.x),
+                                         fma(hud, nu.y, hu * nud.y) + fma(hwd, nv.y, hw * nvd.y));
+        kk[0] += fb.x * Fs.x + fb.y * Fs.y;
+        kk[1] += fb.x * Fb.x + fb.y * Fb.y;
+        double2 c = sm.xd[v];
+        c.x += fma(P.ks, Fsd.x, P.kb * Fbd.x);
+        c.y += fma(P.ks, Fsd.y, P.kb * Fbd.y);
+        if (P.ka != 0.0) {   // F_a = fa (X_{v+1} - X_{v-1}) turned by -90 degrees
+            const double2 d = sm.X[w] - sm.X[u], dd = sm.ext[w] - sm.ext[u];
+            c.x += P.ka * (fad * d.y + fa * dd.y);
+            c.y -= P.ka * (fad * d.x + fa * dd.x);
+        }
+        sm.xd[v] = c;
     }
     block_reduce<2, false>(kk, sm.red);
     if (threadIdx.x == 0) {
@@ -1300,7 +1323,7 @@ lbmib_status reverse_segment(lbmib_ctx* c, long long n0, int len, char* w, const
                                                        (double*)(w + a.fib[r3(n + 1)]),
                                                        (double*)(w + a.bbar[1 - par]), grad + 2 * ncaps);
         if (ncaps > 0)
-            k_adj_membrane<<<ncaps, 128, smem, s>>>(L, c->nd, Xn, c->max_n, Fvs[par], shps[par], fbar, bbar, xnew,
+            k_adj_membrane<<<ncaps, 128, transpose_smem(c->max_n), s>>>(L, c->nd, Xn, c->max_n, Fvs[par], shps[par], fbar, bbar, xnew,
                                                        xc, ncaps, grad);
         c->launches += ncaps > 0 ? 4 : 1;
         LBMIB_CUDA(c, cudaGetLastError());
@@ -1367,7 +1390,7 @@ lbmib_status reverse_segment_dynamic(lbmib_ctx* c, long long n0, int len, char* 
                     pending = true;
                 }
             }
-            k_adjd_update<<<ncaps, 128, smem, s>>>(c->nd, c->max_n, Xn, xc, xm, ub, xout, utb,
+            k_adjd_update<<<ncaps, 128, transpose_smem(c->max_n), s>>>(c->nd, c->max_n, Xn, xc, xm, ub, xout, utb,
                                                    (double2*)(w + a.ftb), ncaps, grad);
             k_adjd_tract<S><<<nblk(2LL * count, kTractGroups), kTractThreads, 0, s>>>(
                 L, c->nd, count, Xn, post1, (const double2*)(w + a.ftb), xout, sb_in, grad + 2 * ncaps,
@@ -1466,9 +1489,9 @@ lbmib_status lbmib_adjoint(lbmib_ctx* c, long long nsteps, lbmib_scheme scheme, 
     if (c->max_n > 0) {
         const int sm_bytes = (int)ring_smem_bytes(c->max_n);
         cudaFuncSetAttribute(k_adj_spread, cudaFuncAttributeMaxDynamicSharedMemorySize, sm_bytes);
-        cudaFuncSetAttribute(k_adj_membrane, cudaFuncAttributeMaxDynamicSharedMemorySize, sm_bytes);
+        cudaFuncSetAttribute(k_adj_membrane, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)transpose_smem(c->max_n));
         cudaFuncSetAttribute(k_adjd_forcing, cudaFuncAttributeMaxDynamicSharedMemorySize, sm_bytes);
-        cudaFuncSetAttribute(k_adjd_update, cudaFuncAttributeMaxDynamicSharedMemorySize, sm_bytes);
+        cudaFuncSetAttribute(k_adjd_update, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)transpose_smem(c->max_n));
     }
     char* w = (char*)d_work;
     cudaStream_t s = c->stream;
