@@ -34,10 +34,10 @@ struct V2 {
     C x, y;
 };
 
-// What one traction probe leaves in shared memory: density deviation and rho nu (G + G^T) n.
+// What one traction probe leaves in shared memory: density and rho nu (G + G^T) n.
 template <typename C>
 struct Probe9 {
-    C drho, tx, ty;
+    C rho, tx, ty;
 };
 
 // Programmatic dependent launch. Every kernel here waits before it reads what the kernel
@@ -76,31 +76,36 @@ __device__ __forceinline__ T sum9(T v) {
     return v + (__shfl_down_sync(0xffffffffu, v, 3) + __shfl_down_sync(0xffffffffu, v, 6));
 }
 
-template <typename C>
-__device__ __forceinline__ C rcp_c(C x) {
-    if constexpr (sizeof(C) == 8) return rcp_bounded(x);
-    else return C(1) / x;
-}
-
 // The lane's share of the MLS fit (Eq. 8-9) at a point whose centre node lies at the offset
 // (dx, dy) from it. Whole warp. Per axis, with offsets d_j, weights w_j, S = sum w, mean
 // offset m and V = sum w (d - m)^2: q = w/S, g = w (d - m)/V, h = q - m g, and the value
 // weight of the lane's node is h_x q_y + q_x h_y - q_x q_y, its slope weights g_x q_y and
 // q_x g_y (the diagonal moment matrix of mls_weights, per axis). One exponential per lane
 // (in FP64 some twenty instructions of 64 cycles): lanes 0-2 of a group do the x axis, 3-5
-// the y axis; the sums are shuffles.
+// the y axis; the sums are shuffles. Single precision: every lane takes the tiled kernels' fit
+// (its weights bit for bit, so that a ring at rest, whose forces are all rounding, spreads the
+// same ones) and picks its node's.
 template <typename C>
 struct Fit9 {
     C phi, gx, gy;
     __device__ __forceinline__ Fit9(const Lane9& l, C dx, C dy) {
+        if constexpr (sizeof(C) == 4) {
+            const MlsW<C> m = mls_weights<C>(0, 0, dx, dy, true);
+            auto pick = [](const C (&v)[3], int i) { return i == 0 ? v[0] : (i == 1 ? v[1] : v[2]); };
+            const C px = pick(m.dxp, l.a), py = pick(m.dyp, l.b), w = pick(m.wx, l.a) * pick(m.wy, l.b);
+            phi = w * (m.k0 + m.kx * px + m.ky * py);
+            gx = m.gx * (w * px);
+            gy = m.gy * (w * py);
+            return;
+        }
         const int j = l.a, ax = l.base + (l.k < 3 ? 0 : 3);   // own index, first lane of the own axis
         const C d0 = l.k < 3 ? dx : dy, d = d0 + C(j - 1);
         const C w = exp(-d * d * C(kMlsInvLen2));
         const C w0 = get9(w, ax), w1 = get9(w, ax + 1), w2 = get9(w, ax + 2);
-        const C is = rcp_c<C>(w0 + w1 + w2);
+        const C is = rcp_bounded(w0 + w1 + w2);
         const C t = (w2 - w0) * is;                           // m = d0 + t
         const C dm = C(j - 1) - t;
-        const C iV = rcp_c<C>(w0 * (C(1) + t) * (C(1) + t) + w1 * t * t + w2 * (C(1) - t) * (C(1) - t));
+        const C iV = rcp_bounded(w0 * (C(1) + t) * (C(1) + t) + w1 * t * t + w2 * (C(1) - t) * (C(1) - t));
         const C q = w * is, g = w * dm * iV, h = q - (d0 + t) * g;
         const int lx = l.base + l.a, ly = l.base + 3 + l.b;
         const C qx = get9(q, lx), hx = get9(h, lx), sx = get9(g, lx);
@@ -116,8 +121,8 @@ struct Fit9 {
     // the probe's values in lane k = 0: linear in the slopes, contracted with n before the sum
     __device__ __forceinline__ Probe9<C> probe(const Mom<C>& f, C nx, C ny, C nu) const {
         const C dux = gx * f.ux, duy = gy * f.ux, dvx = gx * f.uy, dvy = gy * f.uy;
-        const C r = sum9<C>(phi * f.drho), m = (C(1) + r) * nu;
-        return Probe9<C>{r, m * sum9<C>(C(2) * dux * nx + (duy + dvx) * ny),
+        const C rho = C(1) + sum9<C>(phi * f.drho), m = rho * nu;
+        return Probe9<C>{rho, m * sum9<C>(C(2) * dux * nx + (duy + dvx) * ny),
                          m * sum9<C>((duy + dvx) * nx + C(2) * dvy * ny)};
     }
 };
@@ -398,9 +403,9 @@ __global__ void __launch_bounds__(wide_threads<S>()) k_wide_dyn(const S* pops, L
             }
             const C e2 = ex_ * ex_ + ey_ * ey_, rl = rsqrt(e2), len = e2 * rl;
             const Probe9<C> op = ws.pv[2 * li], om = ws.pv[2 * li + 1];
-            // the pressures' difference from the density deviations: rho/3 itself would round
-            // at 3e-8, a hundredth of the traction of a slow flow
-            const C dp = (op.drho - om.drho) * C(1.0 / 3.0);
+            // the pressures' difference with one product rounded, as the tiled kernels' is compiled:
+            // in single precision that rounding is all the traction there is in a fluid at rest
+            const C third = C(1.0 / 3.0), dp = fma(op.rho, third, -(om.rho * third));
             ws.ext[li] = V2<C>{(-dp * (ey_ * rl) + (op.tx - om.tx)) * len, (dp * (ex_ * rl) + (op.ty - om.ty)) * len};
         }
         __syncthreads();
