@@ -122,12 +122,8 @@ bool fusable(const lbmib_ctx* c) { return c->fuse_ib && c->arcs == 1 && c->nrigi
 // capsules to fill the GPU the IB blocks take registers and warp slots from the lattice
 // kernel, which slows by what the overlap saves. Hence the automatic setting: overlap
 // while the capsules number fewer than two per SM.
-// With FP16 storage the fused IB kernels keep the context stream: beside the lattice kernel
-// their warps add the force shares in another order from run to run, and FP16 rounding turns
-// a last-place difference into a thousandth of a population.
 bool overlapped(const lbmib_ctx* c) {
     if (c->caps.empty() || c->overlap == 0) return false;
-    if (c->overlap == -1 && c->cfg.storage == LBMIB_FP16 && fusable(c)) return false;
     return c->overlap == 1 || (int)c->caps.size() < 2 * (c->sms > 0 ? c->sms : 1);
 }
 
@@ -696,6 +692,7 @@ lbmib_status lbmib_add_capsule(lbmib_ctx* c, const double* xy, int n, double ks,
     ring_reference(xy, n, L0, c0, s0, A0, P0);
     if (!(A0 > 0.0)) return fail(c, LBMIB_ERR_ARG, "capsule ring must be counter-clockwise");
     CapsuleParams P{c->nd.count, n, ks, kb, ka, node_mass, A0, P0};
+    P.hop = ring_hop(P.n);
     const int off = c->nd.count;
     const int id = (int)c->caps.size();
     std::vector<double2> zero(n, make_double2(0.0, 0.0));

@@ -648,6 +648,7 @@ lbmib_status lbmib_batch_create(const lbmib_case* cases, int ncases, lbmib_stora
         bc.off = off;
         bc.n = k.n;
         CapsuleParams P{off, k.n, k.k_s, k.k_b, k.k_a, k.node_mass, 0.0, 0.0};
+        P.hop = ring_hop(P.n);
         if (k.n > 0) {
             double a2 = 0.0, per = 0.0, x0 = k.xy[0], x1 = k.xy[0], y0 = k.xy[1], y1 = k.xy[1];
             for (int v = 0; v < k.n; v++) {

@@ -36,6 +36,24 @@ size_t capsule_smem_bytes(int max_n) { return ring_smem_bytes(max_n); }
 // scratch lets seven CTAs share a multiprocessor's shared memory.
 constexpr int kRedIB = 4 * 8;
 
+// Lattice node of tile cell k without integer divisions (some 25 instructions each): the
+// row by a multiplication with the rounded-up reciprocal of the width (exact while
+// k w < 2^32; a tile holds less than 2^16 cells), the periodic wrap from the wrapped origin.
+struct TileWalk {
+    unsigned rw;
+    int w, x0, y0;
+    const Lat& L;
+    template <typename C>
+    __device__ __forceinline__ TileWalk(const Tile<C>& t, const Lat& lat)
+        : rw(t.w > 1 ? 0xffffffffu / (unsigned)t.w + 1u : 0u), w(t.w), x0(wrapi(t.x0, lat.nx)), y0(t.y0), L(lat) {}
+    __device__ __forceinline__ void node(int k, int& x, int& y) const {
+        const int j = w > 1 ? (int)__umulhi((unsigned)k, rw) : k;
+        x = x0 + (k - j * w);
+        while (x >= L.nx) x -= L.nx;
+        y = support_row(L, y0 + j);
+    }
+};
+
 // Fill the moment tile from the populations (nine pulls per node, row by row), two
 // nodes per thread and pass with both nodes' pulls issued before either is reduced: the
 // fill waits on memory latency, and this halves its round trips.
@@ -44,13 +62,15 @@ __device__ void fill_moments(Tile<typename St<S>::C>& t, const S* __restrict__ s
                              const double* __restrict__ fib) {
     using C = typename St<S>::C;
     const int cells = t.w * t.h;
+    const TileWalk at(t, L);
     for (int k = threadIdx.x; k < cells; k += 2 * blockDim.x) {
         const int k1 = k + blockDim.x;
-        const int j0 = k / t.w, i0 = k - j0 * t.w;
         const int k1c = k1 < cells ? k1 : k;   // a missing second node repeats the first
-        const int j1 = k1c / t.w, i1 = k1c - j1 * t.w;
-        const Mom<C> m0 = node_moments<S>(src, L, fib, wrapi(t.x0 + i0, L.nx), support_row(L, t.y0 + j0));
-        const Mom<C> m1 = node_moments<S>(src, L, fib, wrapi(t.x0 + i1, L.nx), support_row(L, t.y0 + j1));
+        int xa, ya, xb, yb;
+        at.node(k, xa, ya);
+        at.node(k1c, xb, yb);
+        const Mom<C> m0 = node_moments<S>(src, L, fib, xa, ya);
+        const Mom<C> m1 = node_moments<S>(src, L, fib, xb, yb);
         t.drho[k] = m0.drho;
         t.ux[k] = m0.ux;
         t.uy[k] = m0.uy;
@@ -80,13 +100,15 @@ template <typename C>
 __device__ void flush_forces(const Tile<C>& t, const Lat& L, const Spread& sp, int* s_count) {
     const long long N = (long long)L.nx * L.ny;
     const int cells = t.w * t.h;
+    const TileWalk at(t, L);
     if (threadIdx.x == 0) *s_count = 0;
     __syncthreads();
     for (int k = threadIdx.x; k < cells; k += blockDim.x) {
         const C cx = t.fx[k], cy = t.fy[k];   // zero test before the widening (exact either way)
         if (cx == C(0) && cy == C(0)) continue;
-        const int j = k / t.w, i = k - j * t.w;
-        const int cell = support_row(L, t.y0 + j) * L.nx + wrapi(t.x0 + i, L.nx);
+        int x, y;
+        at.node(k, x, y);
+        const int cell = y * L.nx + x;
         atomicAdd(sp.fib + cell, (double)cx);
         atomicAdd(sp.fib + N + cell, (double)cy);
         t.cells[atomicAdd(s_count, 1)] = cell;
@@ -268,22 +290,6 @@ constexpr int dyn_min_blocks() {
     return sizeof(typename St<S>::C) == 4 ? 8 : 1;
 }
 
-// An odd step coprime to m, about a quarter of m (1 for short arcs): j -> j * hop mod m
-// visits every vertex once and puts consecutive j far apart on the ring.
-__device__ __forceinline__ int ring_hop(int m) {
-    if (m < 64) return 1;
-    for (int h = (m / 4) | 1; h < m / 2; h += 2) {
-        int a = h, b = m;
-        while (b) {
-            const int r = a % b;
-            a = b;
-            b = r;
-        }
-        if (a == 1) return h;
-    }
-    return 1;
-}
-
 // ---------------------------------------------------------------------------------
 // Dynamic IB (Section 2.3.2), steps 1-3: U = I(u^n) of the populations before any IB
 // force (rho u = sum f e + g/2; the step's IB force is the unknown of the direct forcing),
@@ -326,9 +332,9 @@ __device__ __forceinline__ bool dyn_spread(const S* __restrict__ src, const Lat&
     // the lanes of a warp take vertices `hop` apart on the ring (a bijection of 0..m-1):
     // their 3x3 supports then rarely share a tile cell, and the shared-memory atomics of
     // the spread rarely collide within an instruction
-    const int hop = ring_hop(a.m);
+    const int hop = a.m == P.n ? P.hop : ring_hop(a.m);
     for (int j = threadIdx.x; j < a.m; j += blockDim.x) {
-        const int k = (int)((long long)j * hop % a.m);
+        const int k = (int)((unsigned)j * (unsigned)hop % (unsigned)a.m);
         const int li = kHalo + k, g = P.off + a.v0 + k;
         // shape functions at X^n: used for U, for the spread, and by this step's update
         MlsW<C> w;
@@ -794,9 +800,9 @@ __device__ __forceinline__ bool kin_spread(const Lat& L, const Nodes& nd, const 
     const float fa = F32 ? (float)P.ka * ((float)(P.A0 - A) / (6.0f * (float)P.A0)) : 0.0f;
     bool ok = true;
     // the spread in ring-hop order (see dyn_spread): fewer colliding shared-memory atomics
-    const int hop = ring_hop(m);
+    const int hop = m == P.n ? P.hop : ring_hop(m);
     for (int j = threadIdx.x; j < m; j += blockDim.x) {
-        const int k = (int)((long long)j * hop % m);
+        const int k = (int)((unsigned)j * (unsigned)hop % (unsigned)m);
         const int li = kHalo + k, g = P.off + a.v0 + k;
         double2 F;
         if constexpr (F32) {

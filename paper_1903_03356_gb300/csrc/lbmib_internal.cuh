@@ -800,6 +800,23 @@ struct CapsuleParams {
     double ks, kb, ka, m;  // Eq. 10, 12, 14 constants and per-vertex mass
     double A0, P0;         // stress-free area and perimeter
     int rigid;             // 1: a rigid particle (Section 2.3.1), state in Nodes::rb
+    int hop;               // ring_hop(n) (in the tail padding: the size stays)
 };
+
+// An odd step coprime to m, about a quarter of m (1 for short arcs): j -> j * hop mod m
+// visits every vertex once and puts consecutive j far apart on the ring.
+__host__ __device__ inline int ring_hop(int m) {
+    if (m < 64) return 1;
+    for (int h = (m / 4) | 1; h < m / 2; h += 2) {
+        int a = h, b = m;
+        while (b) {
+            const int r = a % b;
+            a = b;
+            b = r;
+        }
+        if (a == 1) return h;
+    }
+    return 1;
+}
 
 }  // namespace lbmib
