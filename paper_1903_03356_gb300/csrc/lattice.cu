@@ -80,7 +80,7 @@ __device__ __forceinline__ void st_vec(S* p, const typename St<S>::C (&o)[Vec<S>
 // own opposite population) and, for an edge lane, the one scalar that no neighbouring
 // lane holds; resolve() shifts by -e_x through warp shuffles. All 32 lanes of the warp
 // call both with the same y. A chunk that crosses the end of the row ("ragged", only when
-// nx is not a multiple of V) is left to k_ragged: gathered element by element in here, it
+// nx is not a multiple of V) is left to k_nodes: gathered element by element in here, it
 // made its warp three times as long, and with it its block's stay on the multiprocessor
 // (4099 x 2053, FP32: 112 -> 97 us).
 template <typename S, int I, int LM>
@@ -151,9 +151,10 @@ __global__ void __launch_bounds__(BS, MINB) k_collide_stream(const S* __restrict
                                                              Lat L, unsigned* __restrict__ status) {
     using C = typename St<S>::C;
     constexpr int V = Vec<S>::V;
+    asm volatile("griddepcontrol.launch_dependents;");   // k_nodes may start beside the last blocks
     const int lane = threadIdx.x & 31;
     const long long gw = ((long long)blockIdx.x * BS + threadIdx.x) >> 5;
-    const int segs = (L.nx / V + 31) / 32;   // whole vectors only: the rest of a row is k_ragged's
+    const int segs = (L.nx / V + 31) / 32;   // whole vectors only: the rest of a row is k_nodes'
     if (gw >= (long long)segs * L.ny) return;  // whole warps only
     const int y = (int)(gw / segs);
     const int seg = (int)(gw - (long long)y * segs);
@@ -221,9 +222,10 @@ __global__ void __launch_bounds__(BS, MINB) k_collide_stream_d(const double* __r
                                                                double* __restrict__ dst, Lat L, CollideD k,
                                                                unsigned* __restrict__ status) {
     constexpr int V = 2;
+    asm volatile("griddepcontrol.launch_dependents;");   // k_nodes may start beside the last blocks
     const int lane = threadIdx.x & 31;
     const long long gw = ((long long)blockIdx.x * BS + threadIdx.x) >> 5;
-    const int segs = (L.nx / V + 31) / 32;   // whole vectors only: the rest of a row is k_ragged's
+    const int segs = (L.nx / V + 31) / 32;   // whole vectors only: the rest of a row is k_nodes'
     if (gw >= (long long)segs * L.ny) return;  // whole warps only
     const int y = (int)(gw / segs);
     const int seg = (int)(gw - (long long)y * segs);
@@ -433,21 +435,28 @@ __global__ void __launch_bounds__(128) k_ragged_h(const __half* __restrict__ src
     if (ragged_chunk_h(src, dst, L, L.nx / V * V, y, L.gxf, L.gyf, L.omegaf)) atomicOr(status, kStatUnstable);
 }
 
-// The nodes of FP32 and FP64 rows beyond the last whole vector (nx not a multiple of V), one
-// thread per node.
+// FP32 and FP64 nodes from column x0 on, one thread per node: the nodes beyond a row's last
+// whole vector (nx not a multiple of V), beside the vector kernel, or a whole small lattice.
+// Launched as the vector kernel's programmatic dependent: it starts when that kernel's last
+// blocks have, and ends (the wait) after it.
 template <typename S>
-__global__ void __launch_bounds__(128) k_ragged(const S* __restrict__ src, S* __restrict__ dst, Lat L,
-                                                unsigned* __restrict__ status) {
+__global__ void __launch_bounds__(128) k_nodes(const S* __restrict__ src, S* __restrict__ dst, Lat L, int x0,
+                                               CollideD kd, unsigned* __restrict__ status) {
     using C = typename St<S>::C;
-    const int x0 = L.nx / Vec<S>::V * Vec<S>::V, w = L.nx - x0;
-    const int t = blockIdx.x * blockDim.x + threadIdx.x, y = t / w, x = x0 + t - y * w;
-    if (y >= L.ny) return;
-    C s[9];
-    pull_all<S>(src, L, x, y, s);
-    const C usq = collide<C>(s, lat_c<C>(L.gx, L.gxf), lat_c<C>(L.gy, L.gyf), lat_c<C>(L.omega, L.omegaf));
-    if (!(usq < C(0.09))) atomicOr(status, kStatUnstable);
+    const int w = L.nx - x0;
+    const long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+    const int y = (int)(t / w), x = x0 + (int)(t - (long long)y * w);
+    if (y < L.ny) {
+        C s[9];
+        pull_all<S>(src, L, x, y, s);
+        C usq;
+        if constexpr (sizeof(C) == 8) usq = collide_d(s, kd);
+        else usq = collide<C>(s, L.gxf, L.gyf, L.omegaf);
+        if (!(usq < C(0.09))) atomicOr(status, kStatUnstable);
 #pragma unroll
-    for (int i = 0; i < 9; i++) St<S>::st(dst + (long long)i * L.plane + (long long)y * L.pitch + x, s[i], L);
+        for (int i = 0; i < 9; i++) St<S>::st(dst + (long long)i * L.plane + (long long)y * L.pitch + x, s[i], L);
+    }
+    asm volatile("griddepcontrol.wait;" ::: "memory");
 }
 
 // Forced-node patch: the nodes of the current touched-cell list collide with the total
@@ -683,21 +692,42 @@ void launch_collide_stream(const void* src, void* dst, const Lat& L, unsigned* s
             return;
         }
     }
-    if (const int w = L.nx % V) {
-        if constexpr (std::is_same<S, __half>::value) k_ragged_h<V><<<blocks_for(L.ny, 128), 128, 0, s>>>(a, b, L, status);
-        else k_ragged<S><<<blocks_for((long long)L.ny * w, 128), 128, 0, s>>>(a, b, L, status);
+    const int w = L.nx % V;
+    if constexpr (!std::is_same<S, __half>::value) {
+        // A small ragged lattice is one launch of one thread per node: below 2^18 nodes the
+        // second launch costs more than the vectors give.
+        if (w && (long long)L.nx * L.ny <= (1 << 18)) {
+            k_nodes<S><<<blocks_for((long long)L.nx * L.ny, 128), 128, 0, s>>>(a, b, L, 0, CollideD(L.gx, L.gy, L.omega),
+                                                                                status);
+            return;
+        }
     }
-    if (segs == 0) return;
-    if constexpr (std::is_same<S, double>::value) {
-        const CollideD k(L.gx, L.gy, L.omega);
-        if (bs == 256) k_collide_stream_d<256, 3><<<g, 256, 0, s>>>(a, b, L, k, status);
-        else k_collide_stream_d<128, 6><<<g, 128, 0, s>>>(a, b, L, k, status);
-        return;
+    if (segs > 0) {
+        if constexpr (std::is_same<S, double>::value) {
+            const CollideD k(L.gx, L.gy, L.omega);
+            if (bs == 256) k_collide_stream_d<256, 3><<<g, 256, 0, s>>>(a, b, L, k, status);
+            else k_collide_stream_d<128, 6><<<g, 128, 0, s>>>(a, b, L, k, status);
+        } else {
+            if (bs == 256 && !occ4) k_collide_stream<S, 0, 0, 256, 3><<<g, 256, 0, s>>>(a, b, L, status);
+            else if (bs == 256) k_collide_stream<S, 0, 0, 256, 4><<<g, 256, 0, s>>>(a, b, L, status);
+            else if (!occ4) k_collide_stream<S, 0, 0, 128, 6><<<g, 128, 0, s>>>(a, b, L, status);
+            else k_collide_stream<S, 0, 0, 128, 8><<<g, 128, 0, s>>>(a, b, L, status);
+        }
+    }
+    if (w == 0) return;
+    if constexpr (std::is_same<S, __half>::value) {
+        k_ragged_h<V><<<blocks_for(L.ny, 128), 128, 0, s>>>(a, b, L, status);
     } else {
-    if (bs == 256 && !occ4) k_collide_stream<S, 0, 0, 256, 3><<<g, 256, 0, s>>>(a, b, L, status);
-    else if (bs == 256) k_collide_stream<S, 0, 0, 256, 4><<<g, 256, 0, s>>>(a, b, L, status);
-    else if (!occ4) k_collide_stream<S, 0, 0, 128, 6><<<g, 128, 0, s>>>(a, b, L, status);
-    else k_collide_stream<S, 0, 0, 128, 8><<<g, 128, 0, s>>>(a, b, L, status);
+        cudaLaunchConfig_t cfg = {};
+        cfg.gridDim = dim3(blocks_for((long long)L.ny * w, 128));
+        cfg.blockDim = dim3(128);
+        cfg.stream = s;
+        cudaLaunchAttribute at[1];
+        at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+        at[0].val.programmaticStreamSerializationAllowed = 1;
+        cfg.attrs = at;
+        cfg.numAttrs = segs > 0 ? 1 : 0;
+        cudaLaunchKernelEx(&cfg, k_nodes<S>, a, b, L, L.nx - w, CollideD(L.gx, L.gy, L.omega), status);
     }
 }
 
