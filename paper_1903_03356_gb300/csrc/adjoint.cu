@@ -52,7 +52,6 @@ struct Dual {
 __device__ __forceinline__ Dual mk(double v, double d = 0.0) { return Dual{v, d}; }
 __device__ __forceinline__ Dual operator+(Dual a, Dual b) { return {a.v + b.v, a.d + b.d}; }
 __device__ __forceinline__ Dual operator-(Dual a, Dual b) { return {a.v - b.v, a.d - b.d}; }
-__device__ __forceinline__ Dual operator-(Dual a) { return {-a.v, -a.d}; }
 __device__ __forceinline__ Dual operator*(Dual a, Dual b) { return {a.v * b.v, a.d * b.v + a.v * b.d}; }
 __device__ __forceinline__ Dual operator/(Dual a, Dual b) {
     const double q = a.v / b.v;
@@ -382,23 +381,19 @@ __global__ void __launch_bounds__(kInterpThreads) k_adj_interp(Lat L, const S* _
         double q[9];
 #pragma unroll
         for (int i = 0; i < 9; i++) q[i] = (double)qc[i];
-        double drho = 0.0, mx = 0.0, my = 0.0;
-#pragma unroll
-        for (int i = 0; i < 9; i++) {
-            drho += q[i];
-            mx += ex(i) * q[i];
-            my += ey(i) * q[i];
-        }
-        const double rho = 1.0 + drho;
-        const double ux = (mx + 0.5 * (L.gx + fib[cell])) / rho;
-        const double uy = (my + 0.5 * (L.gy + fib[N + cell])) / rho;
+        const double d5 = q[5] - q[7], d6 = q[6] - q[8];
+        const double drho = ((q[0] + (q[1] + q[3])) + (q[2] + q[4])) + ((q[5] + q[7]) + (q[6] + q[8]));
+        const double ir = rcp_newton(1.0 + drho);
+        const double ux = ((q[1] - q[3]) + (d5 - d6) + 0.5 * (L.gx + fib[cell])) * ir;
+        const double uy = ((q[2] - q[4]) + (d5 + d6) + 0.5 * (L.gy + fib[N + cell])) * ir;
         const double uU = ux * Ux + uy * Uy;
         atomicAdd(&xnew[v].x, s.px[b][a] * uU);
         atomicAdd(&xnew[v].y, s.py[b][a] * uU);
-        const double cf = s.phi[b][a] / rho;
+        const double cf = s.phi[b][a] * ir;
+        const double sx = cf * Ux, sy = cf * Uy, sc = -cf * uU, sp = sc + sx, sm = sc - sx;
+        const double share[9] = {sc, sp, sc + sy, sm, sc - sy, sp + sy, sm + sy, sm - sy, sp - sy};
 #pragma unroll
-        for (int i = 0; i < 9; i++)
-            atomicAdd(sbar + (long long)i * N + cell, cf * ((ex(i) - ux) * Ux + (ey(i) - uy) * Uy));
+        for (int i = 0; i < 9; i++) atomicAdd(sbar + (long long)i * N + cell, share[i]);
         atomicAdd(bbar + cell, 0.5 * cf * Ux);
         atomicAdd(bbar + N + cell, 0.5 * cf * Uy);
         gsx = 0.5 * cf * Ux;
@@ -824,37 +819,38 @@ __global__ void __launch_bounds__(128) k_adjd_spread(Lat L, Nodes nd, int max_n,
     }
 }
 
-// Fields (density deviation, velocity before any IB force, density) at lattice node (xk, yk).
+// Fields (density deviation, velocity before any IB force, reciprocal density) at lattice
+// node (xk, yk), by sums and differences of opposite directions.
 template <typename S>
 __device__ __forceinline__ void node_fields(const S* __restrict__ post, const Lat& L, int xk, int yk, double& drho,
-                                            double& ux, double& uy) {
-    double mx = 0.0, my = 0.0;
-    drho = 0.0;
+                                            double& ux, double& uy, double& ir) {
     typename St<S>::C qc[9];
     pull_all<S>(post, L, xk, yk, qc);
+    double q[9];
 #pragma unroll
-    for (int i = 0; i < 9; i++) {
-        const double q = (double)qc[i];
-        drho += q;
-        mx += ex(i) * q;
-        my += ey(i) * q;
-    }
-    const double rho = 1.0 + drho;
-    ux = (mx + 0.5 * L.gx) / rho;
-    uy = (my + 0.5 * L.gy) / rho;
+    for (int i = 0; i < 9; i++) q[i] = (double)qc[i];
+    const double d5 = q[5] - q[7], d6 = q[6] - q[8];
+    drho = ((q[0] + (q[1] + q[3])) + (q[2] + q[4])) + ((q[5] + q[7]) + (q[6] + q[8]));
+    ir = rcp_newton(1.0 + drho);
+    ux = ((q[1] - q[3]) + (d5 - d6) + 0.5 * L.gx) * ir;
+    uy = ((q[2] - q[4]) + (d5 + d6) + 0.5 * L.gy) * ir;
 }
 
 // Adjoint of the fields at support node `cell`: drho-bar and u-bar into the population
-// adjoint (drho = sum s, u = (m + g/2) / rho) and the body-force gradient.
+// adjoint (drho = sum s, u = (m + g/2) / rho, ir = 1/rho) and the body-force gradient. The
+// nine shares differ by e.u-bar/rho only (with a division for each, the two kernels that
+// call this spent a third of their FP64 instructions here).
 __device__ __forceinline__ void inject_fields(const Lat& L, long long cell, double drho_b, double ubx, double uby,
-                                              double ux, double uy, double rho, double* sbar, double& gsx,
+                                              double ux, double uy, double ir, double* sbar, double& gsx,
                                               double& gsy) {
     const long long N = (long long)L.nx * L.ny;
+    const double a = ubx * ir, b = uby * ir, c = drho_b - fma(ux, a, uy * b);
+    const double cp = c + a, cm = c - a;
+    const double share[9] = {c, cp, c + b, cm, c - b, cp + b, cm + b, cm - b, cp - b};
 #pragma unroll
-    for (int i = 0; i < 9; i++)
-        atomicAdd(sbar + (long long)i * N + cell, drho_b + ((ex(i) - ux) * ubx + (ey(i) - uy) * uby) / rho);
-    gsx += 0.5 * ubx / rho;
-    gsy += 0.5 * uby / rho;
+    for (int i = 0; i < 9; i++) atomicAdd(sbar + (long long)i * N + cell, share[i]);
+    gsx += 0.5 * a;
+    gsy += 0.5 * b;
 }
 
 // DR1: transposes of Eq. 24, Eq. 23 and the membrane force, one CTA per capsule. Writes
@@ -917,7 +913,7 @@ __global__ void __launch_bounds__(kTractThreads) k_adjd_tract(Lat L, Nodes nd, i
     bool ok = true;
     int g2 = 0, cx = 0, cy = 0;
     double2 X1{}, X2{};
-    double dx = 0.0, dy = 0.0, len = 1.0, Px = 0.0, Py = 0.0, dr = 0.0, u = 0.0, w = 0.0;
+    double dx = 0.0, dy = 0.0, len = 1.0, rl = 1.0, Px = 0.0, Py = 0.0, dr = 0.0, u = 0.0, w = 0.0, ir = 1.0;
     long long cell = 0;
     R Fb[2] = {R(0), R(0)};
     if (act) {
@@ -931,14 +927,16 @@ __global__ void __launch_bounds__(kTractThreads) k_adjd_tract(Lat L, Nodes nd, i
         Fb[1] = R(0.5 * (f1.y + f2.y));
         dx = X2.x - X1.x;
         dy = X2.y - X1.y;
-        len = sqrt(dx * dx + dy * dy);
+        const double l2 = fma(dx, dx, dy * dy);
+        rl = rsqrt_newton(l2);
+        len = l2 * rl;
         const double sg = s == 0 ? 1.2 : -1.2;
-        Px = 0.5 * (X1.x + X2.x) + sg * dy / len;
-        Py = 0.5 * (X1.y + X2.y) - sg * dx / len;
+        Px = 0.5 * (X1.x + X2.x) + sg * (dy * rl);
+        Py = 0.5 * (X1.y + X2.y) - sg * (dx * rl);
         ok = support_centre(L, Px, Py, cx, cy);
         const int xk = wrapi(cx + k % 3 - 1, L.nx), yk = support_row(L, cy + k / 3 - 1);
         cell = (long long)yk * L.nx + xk;
-        node_fields<S>(post1, L, xk, yk, dr, u, w);
+        node_fields<S>(post1, L, xk, yk, dr, u, w, ir);
         fld[0][grp][k] = R(dr);
         fld[1][grp][k] = R(u);
         fld[2][grp][k] = R(w);
@@ -961,7 +959,7 @@ __global__ void __launch_bounds__(kTractThreads) k_adjd_tract(Lat L, Nodes nd, i
         }
         // fields: dT/drho and dT/dG contracted with F_l-bar, for this thread's node
         const double sgn = s == 0 ? 1.0 : -1.0;
-        const R nn[2] = {R(dy / len), R(-dx / len)};
+        const R nn[2] = {R(dy * rl), R(-dx * rl)};
         const R d0x = R(cx - Px), d0y = R(cy - Py);
         const ProbeVal<R> o = probe_eval<R, R>(d0x, d0y, drho, ux, uy);
         const R lsg = R(sgn * len), nu = R(L.nu);
@@ -982,7 +980,7 @@ __global__ void __launch_bounds__(kTractThreads) k_adjd_tract(Lat L, Nodes nd, i
         const R phi = hxa * qyb + qxa * hyb - qxa * qyb;
         const R gx = gxa * qyb, gy = qxa * gyb;
         inject_fields(L, cell, (double)(phi * rho_b), (double)(Gb[0][0] * gx + Gb[0][1] * gy),
-                      (double)(Gb[1][0] * gx + Gb[1][1] * gy), (double)R(u), (double)R(w), 1.0 + (double)R(dr), sbar,
+                      (double)(Gb[1][0] * gx + Gb[1][1] * gy), u, w, ir, sbar,
                       gsx, gsy);
     }
     for (int o = 16; o > 0; o >>= 1) {
@@ -1011,13 +1009,13 @@ __global__ void __launch_bounds__(kInterpThreads) k_adjd_interp(Lat L, const S* 
         const int a = k % 3, b = k / 3;
         const Shape& s = shp[v];
         const int xk = wrapi(s.cx + a - 1, L.nx), yk = support_row(L, s.cy + b - 1);
-        double drho, ux, uy;
-        node_fields<S>(post, L, xk, yk, drho, ux, uy);
+        double drho, ux, uy, ir;
+        node_fields<S>(post, L, xk, yk, drho, ux, uy, ir);
         const double uU = ux * U.x + uy * U.y;
         atomicAdd(&xout[v].x, s.px[b][a] * uU);
         atomicAdd(&xout[v].y, s.py[b][a] * uU);
         const double phi = s.phi[b][a];
-        inject_fields(L, (long long)yk * L.nx + xk, 0.0, phi * U.x, phi * U.y, ux, uy, 1.0 + drho, sbar, gsx, gsy);
+        inject_fields(L, (long long)yk * L.nx + xk, 0.0, phi * U.x, phi * U.y, ux, uy, ir, sbar, gsx, gsy);
     }
     for (int o = 16; o > 0; o >>= 1) {
         gsx += __shfl_xor_sync(0xffffffffu, gsx, o);
@@ -1063,11 +1061,11 @@ __global__ void __launch_bounds__(128) k_adjd_forcing(Lat L, Nodes nd, int max_n
                 gyv += s.py[b][a] * tF;
             }
         const double2 Xv = sm.X[v], Xl = sm.X[v == 0 ? n - 1 : v - 1], Xr = sm.X[v + 1 == n ? 0 : v + 1];
-        const double ll = sqrt((Xv.x - Xl.x) * (Xv.x - Xl.x) + (Xv.y - Xl.y) * (Xv.y - Xl.y));
-        const double lr = sqrt((Xr.x - Xv.x) * (Xr.x - Xv.x) + (Xr.y - Xv.y) * (Xr.y - Xv.y));
-        const double cl = 0.5 * (ll + lr);
+        const double2 dl = Xv - Xl, dr = Xr - Xv;
+        const double ll2 = fma(dl.x, dl.x, dl.y * dl.y), lr2 = fma(dr.x, dr.x, dr.y * dr.y);
+        const double cl = 0.5 * fma(ll2, rsqrt_newton(ll2), lr2 * rsqrt_newton(lr2));
         // c-bar = F_l . (cF)-bar = (c F_l) . (cF)-bar / c;  F_l-bar = c (cF)-bar
-        sm.sst[v] = (F.x * cfx + F.y * cfy) / cl;
+        sm.sst[v] = (F.x * cfx + F.y * cfy) * rcp_newton(cl);
         sm.ext[v] = make_double2(cl * cfx, cl * cfy);
         const double2 c = xout[g];
         sm.xd[v] = make_double2(c.x + gxv, c.y + gyv);
@@ -1078,9 +1076,9 @@ __global__ void __launch_bounds__(128) k_adjd_forcing(Lat L, Nodes nd, int max_n
         const int vl = v == 0 ? n - 1 : v - 1, vr = v + 1 == n ? 0 : v + 1;
         const double2 Xv = sm.X[v], Xl = sm.X[vl], Xr = sm.X[vr];
         const double dlx = Xv.x - Xl.x, dly = Xv.y - Xl.y, drx = Xr.x - Xv.x, dry = Xr.y - Xv.y;
-        const double ll = sqrt(dlx * dlx + dly * dly), lr = sqrt(drx * drx + dry * dry);
+        const double il = rsqrt_newton(fma(dlx, dlx, dly * dly)), ir = rsqrt_newton(fma(drx, drx, dry * dry));
         // c_u = (l_{u-1} + l_u)/2: X_v gets (d_{v-1}/l_{v-1})(c_v + c_{v-1})/2 - (d_v/l_v)(c_v + c_{v+1})/2
-        const double wl = 0.5 * (sm.sst[v] + sm.sst[vl]) / ll, wr = 0.5 * (sm.sst[v] + sm.sst[vr]) / lr;
+        const double wl = 0.5 * (sm.sst[v] + sm.sst[vl]) * il, wr = 0.5 * (sm.sst[v] + sm.sst[vr]) * ir;
         double2 acc = sm.xd[v];
         acc.x += wl * dlx - wr * drx;
         acc.y += wl * dly - wr * dry;
