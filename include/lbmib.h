@@ -243,16 +243,18 @@ enum { LBMIB_FIELD_POPULATIONS = 0, LBMIB_FIELD_FORCE = 1 };
 lbmib_status lbmib_field_ptr(lbmib_ctx* ctx, int field, void** ptr, int* pitch);
 
 /* Options (lbmib_set_option):
- *   LBMIB_OPT_GRAPHS        1 (default): replay steps from captured CUDA graphs;
- *                           0: launch kernels directly.
+ *   LBMIB_OPT_GRAPHS        1 (default): replay steps from captured CUDA graphs (the
+ *                           steps a call leaves over are captured when a call leaves the
+ *                           same number twice in a row); 0: launch kernels directly.
  *   LBMIB_OPT_TIMING        1: record CUDA events around every lattice-update launch
  *                           (forces direct launches); read with lbmib_kernel_time.
  *   LBMIB_OPT_GRAPH_STEPS   steps per captured graph (default 64; each graph opens with
  *                           its own force and spread and closes with its own update).
  *   LBMIB_OPT_FP16_SCALE    log2 of the FP16 storage scale (default 10).
  *   LBMIB_OPT_LATTICE_VARIANT launch shape of the lattice-update kernel: bits 0-11 the
- *                           block size (128 or 256), bit 18 a 64-register cap (eight
- *                           128-thread or four 256-thread blocks resident per SM), bit 19 (FP16
+ *                           block size (128 or 256), bit 18 (FP32 and FP16 storage) a
+ *                           64-register cap (eight 128-thread or four 256-thread blocks
+ *                           resident per SM), bit 19 (FP16
  *                           storage) the kernel that moves 8 nodes per thread as packed
  *                           16-byte vectors. Default: 128 threads, with the cap for
  *                           FP32/FP16 storage and bit 19 for FP16. Results do not

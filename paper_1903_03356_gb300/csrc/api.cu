@@ -104,6 +104,12 @@ void drop_graphs(lbmib_ctx* c) {
                     cudaGraphExecDestroy(g);
                     g = nullptr;
                 }
+    for (auto& a : c->rest)
+        for (auto& b : a)
+            for (auto& r : b) {
+                if (r.exec) cudaGraphExecDestroy(r.exec);
+                r = lbmib_ctx::RestGraph{};
+            }
 }
 
 // Whether the Dynamic node update of a step may also do the force and spread of the next
@@ -865,9 +871,36 @@ lbmib_status lbmib_step(lbmib_ctx* c, long long nsteps, lbmib_scheme scheme) {
             }
             left -= G;
         }
-        fork_ib(c, c->stream);
-        enqueue_steps(c, scheme, left, c->cur, c->cur_fib, c->stream, false);
-        join_ib(c, c->stream);
+        // The rest of the call. Launched one by one, its kernels' streams are joined by events
+        // through the host's queue: 52 instead of 30 us per step with 256 FP16 capsules.
+        if (left > 0) {
+            lbmib_ctx::RestGraph& r = c->rest[sc][c->cur][c->cur_fib];
+            // a caller that captures the stream itself gets plain launches, as ever
+            cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
+            if (cudaStreamIsCapturing(c->stream, &cs) != cudaSuccess) cudaGetLastError();
+            const bool plain = cs != cudaStreamCaptureStatusNone;
+            if (!plain && left > 1 && r.seen == left && !(r.exec && r.len == left)) {
+                cudaGraphExec_t g = nullptr;
+                lbmib_status st = capture(c, scheme, c->cur, c->cur_fib, (int)left, &g, &r.kernels);
+                if (st != LBMIB_OK) return st;
+                if (r.exec) cudaGraphExecDestroy(r.exec);
+                r.exec = g;
+                r.len = (int)left;
+            }
+            r.seen = (int)left;
+            if (!plain && r.exec && r.len == left) {
+                LBMIB_CUDA(c, cudaGraphLaunch(r.exec, c->stream));
+                c->launches += r.kernels;
+                if (left & 1) {
+                    if (!c->caps.empty()) c->cur_fib = 1 - c->cur_fib;
+                    c->cur = 1 - c->cur;
+                }
+            } else {
+                fork_ib(c, c->stream);
+                enqueue_steps(c, scheme, left, c->cur, c->cur_fib, c->stream, false);
+                join_ib(c, c->stream);
+            }
+        }
     }
     c->steps += nsteps;
     LBMIB_CUDA(c, cudaGetLastError());

@@ -88,6 +88,14 @@ struct lbmib_ctx {
     cudaGraphExec_t graphs[2][2][2]{};
     int graph_len[2][2][2]{};
     long long graph_kernels[2][2][2]{};
+    // the steps a call leaves over (fewer than graph_steps): captured when a call leaves the
+    // same number twice in a row from the same buffers, one graph per (scheme, cur, cur_fib)
+    struct RestGraph {
+        cudaGraphExec_t exec = nullptr;
+        int len = 0, seen = 0;
+        long long kernels = 0;
+    };
+    RestGraph rest[2][2][2]{};
     // timing
     std::vector<std::pair<cudaEvent_t, cudaEvent_t>> ev_pool;
     size_t ev_used = 0;

@@ -128,6 +128,37 @@ def test_paths_alternate_and_states_load(L):
     agree(c, b, case, 1e-12)
 
 
+@pytest.mark.parametrize("scheme", [o.KINEMATIC, o.DYNAMIC])
+@pytest.mark.parametrize("general", [False, True])
+def test_repeated_rests_of_calls(L, scheme, general):
+    # calls that leave the same number of steps over replay a captured rest; others do not
+    case = rings((64, 31))
+    a, b = pair(L, case, "fp64", OPT_OVERLAP=1 if general else -1)
+    if not general:
+        b.set_option(L.OPT_OVERLAP, -1)
+    b.set_option(L.OPT_GRAPHS, 0)
+    n0 = a.launch_count, b.launch_count
+    for n in (5, 5, 5, 7, 5, 11, 11, 11, 1, 1, 4):
+        a.step(n, scheme)
+        b.step(n, scheme)
+    agree(a, b, case, 1e-12)
+    assert a.launch_count - n0[0] >= b.launch_count - n0[1]   # graphs of 8 close and open their own spreads
+
+
+@pytest.mark.parametrize("storage", ["fp64", "fp32", "fp16"])
+@pytest.mark.parametrize("nx, ny", [(3, 5), (5, 40), (259, 33), (1027, 301)])
+def test_ragged_lattices(L, storage, nx, ny):
+    # rows that no vector fits: one thread per node below 2^18 nodes, beside the vector kernel above
+    case = W.Case("ragged", nx, ny, 0.7, True, -0.02, 0.02, gx=1e-5, init="shear")
+    ctx = L.from_case(case, storage=storage)
+    ctx.step(9, o.KINEMATIC)
+    s = o.Sim(o.lattice(nx, ny, 0.7, True, -0.02, 0.02, 1e-5, 0.0))
+    s.init_fields(*case.fields())
+    s.step(9, o.KINEMATIC)
+    tol = {"fp64": 1e-15, "fp32": 5e-9, "fp16": 1e-4}[storage]   # rounding of nine steps of |f - w| < 1e-2
+    np.testing.assert_allclose(ctx.read_populations(), s.populations(), rtol=0, atol=tol)
+
+
 def test_support_error_is_reported(L):
     case = rings((64,))
     ctx = L.from_case(case, storage="fp32")
