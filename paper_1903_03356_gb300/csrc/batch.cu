@@ -133,7 +133,8 @@ __device__ __forceinline__ void tile_force(const Tile<C>& t, const Lat& L, int x
 }
 
 template <typename S>
-__device__ void run_case(const BatchDev& d, int c, int nsteps, const CapSmem& sm, int tile_cells, int max_n) {
+__device__ void run_case(const BatchDev& d, int c, int nsteps, const CapSmem& sm, int tile_cells, int max_n,
+                         int2* centre) {
     using C = typename St<S>::C;
     BatchCase bc = d.cases[c];
     const Lat& L = bc.L;
@@ -176,49 +177,78 @@ __device__ void run_case(const BatchDev& d, int c, int nsteps, const CapSmem& sm
                 for (int v = threadIdx.x; v < n; v += blockDim.x)
                     vertex_terms_f(sm, P, d.nd, v == 0 ? n - 1 : v - 1, v, v + 1 == n ? 0 : v + 1, off + v);
                 __syncthreads();
-                float area2[1] = {0.0f};
-                const double2 X0 = sm.X[0];
-                for (int v = threadIdx.x; v < n; v += blockDim.x) {
-                    const double2 Xv = sm.X[v];
-                    const float2 e = ring_f(sm)[v].e;
-                    area2[0] += (float)(Xv.x - X0.x) * e.y - (float)(Xv.y - X0.y) * e.x;
+                if (P.ka != 0.0) {   // the enclosed area enters only Eq. 14
+                    float area2[1] = {0.0f};
+                    const double2 X0 = sm.X[0];
+                    for (int v = threadIdx.x; v < n; v += blockDim.x) {
+                        const double2 Xv = sm.X[v];
+                        const float2 e = ring_f(sm)[v].e;
+                        area2[0] += (float)(Xv.x - X0.x) * e.y - (float)(Xv.y - X0.y) * e.x;
+                    }
+                    block_reduce<1, false>(area2, sm.red, (n + 31) >> 5);
+                    // Eq. 14 factor k_a (1 - A/A0) p_ref / 2 from the difference A0 - A
+                    fa = (float)P.ka * (((float)P.A0 - 0.5f * area2[0]) / (6.0f * (float)P.A0));
                 }
-                block_reduce<1, false>(area2, sm.red);
-                // Eq. 14 factor k_a (1 - A/A0) p_ref / 2 from the difference A0 - A
-                fa = (float)P.ka * (((float)P.A0 - 0.5f * area2[0]) / (6.0f * (float)P.A0));
             } else {
                 double area2[1] = {0.0};
                 for (int v = threadIdx.x; v < n; v += blockDim.x) area2[0] += ring_terms(sm, P, d.nd, v);
                 block_reduce<1, false>(area2, sm.red);
                 A = 0.5 * area2[0];
             }
+            // Single precision: the forces and support frames of all vertices first, into the slots
+            // the float terms leave unused, then one thread per (support node, vertex) for the
+            // spread: two shared float additions (compare-and-swap loops) in a thread instead
+            // of eighteen, over the whole block instead of one thread per vertex.
             for (int v = threadIdx.x; v < n; v += blockDim.x) {
                 double2 F;
                 if constexpr (F32) {
                     const float2 Ff = internal_force_f(sm, v == 0 ? n - 1 : v - 1, v, v + 1 == n ? 0 : v + 1, fa);
                     F = make_double2(Ff.x, Ff.y);
+                    reinterpret_cast<float2*>(sm.sst)[v] = Ff;
+                    const double2 X = sm.X[v];
+                    double x = X.x, y = X.y;
+                    int cx, cy;
+                    const bool in = support_centre(L, x, y, cx, cy);
+                    centre[v] = make_int2(cx, cy);
+                    reinterpret_cast<float2*>(sm.bs)[v] = make_float2((float)((double)cx - x), (float)((double)cy - y));
+                    if (t.use) ok &= in && t.holds(cx, cy);
                 } else {
                     F = node_internal_force(sm, P, v, A);
-                }
-                if (t.use) {
-                    const MlsW<C> m = mls_setup<C>(L, sm.X[v].x, sm.X[v].y);
-                    ok &= m.ok && t.holds(m.cx, m.cy);
-                    if (t.holds(m.cx, m.cy)) {
-                        const C Fx = C(F.x), Fy = C(F.y);
+                    if (t.use) {
+                        const MlsW<C> m = mls_setup<C>(L, sm.X[v].x, sm.X[v].y);
+                        ok &= m.ok && t.holds(m.cx, m.cy);
+                        if (t.holds(m.cx, m.cy)) {
 #pragma unroll
-                        for (int b = 0; b < 3; b++)
+                            for (int b = 0; b < 3; b++)
 #pragma unroll
-                            for (int a = 0; a < 3; a++) {
-                                const C phi = m.phi(a, b);
-                                const int k = t.index(m.cx + a - 1, m.cy + b - 1);
-                                atomicAdd(t.fx + k, phi * Fx);
-                                atomicAdd(t.fy + k, phi * Fy);
-                            }
+                                for (int a = 0; a < 3; a++) {
+                                    const C phi = m.phi(a, b);
+                                    const int k = t.index(m.cx + a - 1, m.cy + b - 1);
+                                    atomicAdd(t.fx + k, phi * C(F.x));
+                                    atomicAdd(t.fy + k, phi * C(F.y));
+                                }
+                        }
                     }
                 }
                 if (step == nsteps - 1) d.nd.Fint[off + v] = F;
             }
             __syncthreads();
+            if constexpr (F32) {
+                for (int q = threadIdx.x; q < (t.use ? 9 * n : 0); q += blockDim.x) {
+                    const int k = q / n, v = q - k * n;
+                    const int2 c = centre[v];
+                    if (!t.holds(c.x, c.y)) continue;
+                    const float2 d0 = reinterpret_cast<const float2*>(sm.bs)[v], F = reinterpret_cast<const float2*>(sm.sst)[v];
+                    const MlsW<C> m = mls_weights<C>(c.x, c.y, d0.x, d0.y, true);
+                    auto pick = [](const C (&w)[3], int i) { return i == 0 ? w[0] : (i == 1 ? w[1] : w[2]); };
+                    const int a = k % 3, b = k / 3;
+                    const C phi = pick(m.wx, a) * pick(m.wy, b) * (m.k0 + m.kx * pick(m.dxp, a) + m.ky * pick(m.dyp, b));
+                    const int cell = t.index(c.x + a - 1, c.y + b - 1);
+                    atomicAdd(t.fx + cell, phi * F.x);
+                    atomicAdd(t.fy + cell, phi * F.y);
+                }
+                __syncthreads();
+            }
         }
         // iv-vi: the lattice update of the whole case, with the membrane force inline. Each
         // thread walks nodes tid, tid + B, ... keeping (x, y) by carries instead of divisions.
@@ -291,7 +321,13 @@ __device__ void run_case(const BatchDev& d, int c, int nsteps, const CapSmem& sm
             __syncthreads();
             for (int v = threadIdx.x; v < n; v += blockDim.x) {
                 const double2 Xv = sm.X[v];
-                const MlsW<C> m = mls_setup<C>(L, Xv.x, Xv.y);
+                MlsW<C> m;
+                if constexpr (sizeof(C) == 4) {   // the frame the spread left
+                    const float2 d0 = reinterpret_cast<const float2*>(sm.bs)[v];
+                    m = mls_weights<C>(centre[v].x, centre[v].y, d0.x, d0.y, true);
+                } else {
+                    m = mls_setup<C>(L, Xv.x, Xv.y);
+                }
                 InterpT<C> o;
                 if (t.holds(m.cx, m.cy)) {
                     mls_apply<C, false>(m, [&](int a, int b) {
@@ -338,6 +374,8 @@ __device__ void run_case(const BatchDev& d, int c, int nsteps, const CapSmem& sm
     }
 }
 
+__host__ __device__ inline size_t up8(size_t v) { return (v + 7) / 8 * 8; }
+
 template <typename S, int BS>
 __global__ void __launch_bounds__(BS, 1024 / BS) k_batch(BatchDev d, int nsteps, int tile_cells, int max_n) {
     extern __shared__ __align__(16) unsigned char smem[];
@@ -349,13 +387,14 @@ __global__ void __launch_bounds__(BS, 1024 / BS) k_batch(BatchDev d, int nsteps,
         const int q = s_next;
         __syncthreads();
         if (q >= d.ncases) break;
-        run_case<S>(d, d.order[q], nsteps, sm, tile_cells, max_n);
+        run_case<S>(d, d.order[q], nsteps, sm, tile_cells, max_n,
+                    reinterpret_cast<int2*>(sm.tile + up8((size_t)tile_cells * 5 * sizeof(typename St<S>::C))));
     }
 }
 
 template <typename C>
 static size_t batch_smem(int max_n, int cells) {
-    return ring_smem_bytes(max_n) + (size_t)cells * (3 * sizeof(C) + 2 * sizeof(C));
+    return ring_smem_bytes(max_n) + up8((size_t)cells * 5 * sizeof(C)) + (sizeof(C) == 4 ? (size_t)max_n * sizeof(int2) : 0);
 }
 
 template <typename S>

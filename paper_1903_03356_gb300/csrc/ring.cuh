@@ -42,11 +42,12 @@ __device__ __forceinline__ CapSmem carve(unsigned char* base, int max_n, int red
 
 // Reduction of K doubles or floats over the block (blockDim.x a multiple of 32, <= 1024);
 // MIN selects minimum instead of sum. Every thread receives the results. `red_` is the
-// block's double scratch (8 doubles per warp).
+// block's double scratch (8 doubles per warp). Only the first `warps` warps' values count
+// (a short ring fills few of a large block's warps).
 template <int K, bool MIN, typename T>
-__device__ void block_reduce(T (&v)[K], double* red_) {
+__device__ void block_reduce(T (&v)[K], double* red_, int warps = 32) {
     T* red = reinterpret_cast<T*>(red_);
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = min((int)blockDim.x >> 5, warps);
 #pragma unroll
     for (int k = 0; k < K; k++)
         for (int o = 16; o > 0; o >>= 1) {
@@ -112,7 +113,7 @@ __device__ Tile<C> make_tile(const CapSmem& sm, int lo, int hi, int margin, int 
         r[2] = fminf(r[2], -x);
         r[3] = fminf(r[3], -y);
     }
-    block_reduce<4, true>(r, sm.red);
+    block_reduce<4, true>(r, sm.red, max(1, (hi - lo + 31) >> 5));
     Tile<C> t;
     const bool sane = fabsf(r[0]) < kLimit && fabsf(r[1]) < kLimit && fabsf(r[2]) < kLimit && fabsf(r[3]) < kLimit;
     t.x0 = sane ? (int)floorf(r[0]) - margin : 0;
