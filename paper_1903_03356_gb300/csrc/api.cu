@@ -356,7 +356,7 @@ bool enqueue_step(lbmib_ctx* c, lbmib_scheme scheme, int& cur, int& cur_fib, cud
         if (scheme == LBMIB_DYNAMIC) {
             with_ib_storage(c, [&](auto v) {
                 launch_dyn_update<decltype(v)>(dst, L, c->nd, ncaps, c->max_n, c->arcs, c->tile_cells,
-                                               c->nrigid > 0, reset, status, s);
+                                               c->nrigid, reset, status, s);
             });
         } else {
             with_ib_storage(c, [&](auto v) {

@@ -1126,12 +1126,13 @@ void launch_dyn_force_spread(const void* src, const Lat& L, Nodes nd, int ncaps,
 
 template <typename S>
 void launch_dyn_update(const void* dst, const Lat& L, Nodes nd, int ncaps, int max_n,
-                       int arcs, int cells, bool rigid, int* reset_count, unsigned* status, cudaStream_t s) {
+                       int arcs, int cells, int rigid, int* reset_count, unsigned* status, cudaStream_t s) {
     using C = typename St<S>::C;
     const size_t sh = smem_bytes<C>(arc_slots(max_n, arcs), cells, true, false);
-    launch_arcs(k_dyn_update<S>, ncaps, arcs, true, sh, s, (const S*)dst, L, nd, max_n, arcs, cells,
-                reset_count, status);
-    if (rigid)
+    if (rigid < ncaps)   // with rigid particles alone it would only be 6 us of idle CTAs
+        launch_arcs(k_dyn_update<S>, ncaps, arcs, true, sh, s, (const S*)dst, L, nd, max_n, arcs, cells,
+                    reset_count, status);
+    if (rigid > 0)
         launch_arcs(k_rigid_update<S>, ncaps, arcs, true, sh, s, (const S*)dst, L, nd, max_n, arcs, cells,
                     status);
 }
@@ -1189,7 +1190,7 @@ void launch_interp_points(const void* src, const Lat& L, const double* fib, cons
 #define LBMIB_INSTANTIATE_IB(S)                                                                              \
     template void launch_dyn_force_spread<S>(const void*, const Lat&, Nodes, int, int, int, int, bool,       \
                                              Spread, unsigned*, cudaStream_t);                               \
-    template void launch_dyn_update<S>(const void*, const Lat&, Nodes, int, int, int, int, bool, int*,       \
+    template void launch_dyn_update<S>(const void*, const Lat&, Nodes, int, int, int, int, int, int*,        \
                                        unsigned*, cudaStream_t);                                             \
     template void launch_dyn_update_spread<S>(const void*, const Lat&, Nodes, int, int, int, Spread,         \
                                               unsigned*, cudaStream_t);                                      \

@@ -93,11 +93,10 @@ __host__ __device__ inline int arc_slots(int max_n, int arcs) { return (max_n + 
 template <typename S>
 void launch_dyn_force_spread(const void* src, const Lat& L, Nodes nd, int ncaps, int max_n,
                              int arcs, int cells, bool rigid, Spread sp, unsigned* status, cudaStream_t s);
-// the node update of the capsules, then (rigid: the context holds rigid particles) that
-// of the rigid particles
+// the node update of the capsules, then that of the `rigid` rigid particles among them
 template <typename S>
 void launch_dyn_update(const void* dst, const Lat& L, Nodes nd, int ncaps, int max_n,
-                       int arcs, int cells, bool rigid, int* reset_count, unsigned* status, cudaStream_t s);
+                       int arcs, int cells, int rigid, int* reset_count, unsigned* status, cudaStream_t s);
 // the node update of step n and the force and spread of step n+1 in one kernel (one CTA
 // per capsule, no rigid particles), spreading through sp_next
 template <typename S>
