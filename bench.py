@@ -380,7 +380,7 @@ def run_gpu(a):
             "ib_update_ms": ib_ms / ib_n, "ib_update_share": ib_ms / timed_ms,
             "note": ("CUDA events on the context stream around each step's patch (k_patch) and "
                      "immersed-boundary node update (k_dyn_update_spread: the update fused with the "
-                     "next step's force and spread, with the list-counter reset before it); the "
+                     "next step's force and spread); the "
                      "patch's algorithmic bytes per listed node are its 9 populations read and "
                      "written, the 16-byte force read, the last force cleared and three 4-byte "
                      "list and claim words"),

@@ -580,7 +580,7 @@ inline size_t transpose_smem(int max_n) {
 //   angle:   g = sin(theta - theta_0) = (c0 a x b - s0 a.b) r_a r_b, g' likewise
 //   vertex:  F_s = T_v - T_{v-1},  F_b = (g_v - g_{v-1}) n_{v-1} + (g_v - g_{v+1}) n_v,
 // about 90 of them per vertex (as dual numbers over the five-vertex stencil some 650: the
-// Dynamic update transpose of one 128-vertex ring 23.9 -> 8 us).
+// Dynamic update transpose of one 128-vertex ring 23.9 -> 10.9 us).
 __device__ void membrane_transpose(const CapSmem& sm, const CapsuleParams& P, const Nodes& nd, int cap, int ncaps,
                                    double* grad) {
     const int n = P.n, off = P.off;

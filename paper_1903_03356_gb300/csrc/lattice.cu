@@ -82,7 +82,7 @@ __device__ __forceinline__ void st_vec(S* p, const typename St<S>::C (&o)[Vec<S>
 // call both with the same y. A chunk that crosses the end of the row ("ragged", only when
 // nx is not a multiple of V) is left to k_nodes: gathered element by element in here, it
 // made its warp three times as long, and with it its block's stay on the multiprocessor
-// (4099 x 2053, FP32: 112 -> 97 us).
+// (4099 x 2053, FP32: 112 -> 95 us per step).
 template <typename S, int I, int LM>
 struct PopLoad {
     using C = typename St<S>::C;

@@ -14,7 +14,7 @@
 //     probe places, shape functions) is done before griddepcontrol.wait, beside the lattice
 //     kernel (programmatic dependent launch).
 // Per step, tiled kernels against these: 100 x 100 shear box, 64 vertices, Kinematic, FP64
-// 42.8 -> 18.3 us; 360 x 120 open channel, 586 vertices, Dynamic, FP32 27.4 -> 16.2 us.
+// 42.8 -> 18.0 us; 360 x 120 open channel, 586 vertices, Dynamic, FP32 27.4 -> 16.4 us.
 #include <cooperative_groups.h>
 
 #include <algorithm>
