@@ -266,8 +266,8 @@ lbmib_status lbmib_field_ptr(lbmib_ctx* ctx, int field, void** ptr, int* pitch);
  *                           (default): on while there are fewer than two capsules per
  *                           multiprocessor, and small contexts (up to 2^20 nodes and
  *                           32768 vertices, 8192 with FP64 interpolations, no rigid
- *                           particles; in single precision rings of more than a warp per
- *                           CTA) step with two kernels on the context stream, the node
+ *                           particles, not FP16 storage; with FP32 interpolations rings
+ *                           of more than a warp per CTA) step with two kernels on the context stream, the node
  *                           update with the next spread and the lattice update with the
  *                           force in place, when OPT_ARCS and OPT_FUSE_IB are at their
  *                           defaults and OPT_TIMING is off. Results do not depend on it

@@ -171,11 +171,17 @@ void with_ib_storage(const lbmib_ctx* c, F&& f) {
 //    than the tiles' chain;
 //  - in single precision only where a tiled arc is longer than a warp: shorter arcs add
 //    their float shares in a fixed order, so that a tiled run repeats bit for bit, and
-//    positions, which add up every step's rounding, would part from it by 1e-9 in 200 steps.
+//    positions, which add up every step's rounding, would part from it by 1e-9 in 200 steps;
+//  - never with FP16 storage: it rounds a population of 1e-2 to 5e-6, so a force that differs in
+//    its last place, as the shares of the two paths do at every node, moves one population in a
+//    few thousand by such a step, and after 40 steps with 60 capsules on 900 x 500 the
+//    populations of the two paths were 1.3e-4 of their norm apart (the tiled kernels repeat
+//    themselves to 1e-6, and with FP64 interpolations bit for bit).
 bool wide(const lbmib_ctx* c) {
     constexpr long long kWideNodes = 1 << 20, kWideVerts = 32768;
     const bool fp64 = c->cfg.storage == LBMIB_FP64 || c->ib_fp64;
-    if (c->caps.empty() || c->nrigid > 0 || !c->fuse_ib || c->timing || c->overlap != -1 || c->arcs_opt != 0)
+    if (c->caps.empty() || c->nrigid > 0 || !c->fuse_ib || c->timing || c->overlap != -1 || c->arcs_opt != 0 ||
+        c->cfg.storage == LBMIB_FP16)
         return false;
     if (!fp64 && (c->max_n + c->arcs - 1) / c->arcs <= 32) return false;
     return (long long)c->cfg.nx * c->cfg.ny <= kWideNodes && c->nd.count <= (fp64 ? kWideVerts / 4 : kWideVerts) &&
@@ -205,20 +211,25 @@ void enqueue_wide(lbmib_ctx* c, lbmib_scheme scheme, long long n, int& cur, int&
             c->launches += 2;
         }
         auto ib = [&](bool upd, bool spr, const void* pops, int to, double2* tape_x, bool pdl) {
-            with_ib_storage(c, [&](auto v) {
+            auto go = [&](auto v) {
                 launch_wide<decltype(v)>(dyn, upd, spr, pops, L, nd, ncaps, c->max_n, arcs, c->fib[fc], c->fib[to],
                                          c->list[to], &c->ctr->count[to], status, tape_x, pdl, s);
-            });
+            };
+            if (c->cfg.storage == LBMIB_FP64) go(double{});
+            else if (c->ib_fp64) go(f32w{});
+            else go(float{});
             c->launches++;
         };
         if (!spread_done) {
             nd.Flc = tape && tape->flc ? tape->flc + k * tape->nodes : nullptr;
             ib(false, true, src, fc, nullptr, false);
         }
-        by_storage(c->cfg.storage, [&](auto tag) {
+        auto lattice = [&](auto tag) {
             launch_collide_forced<decltype(tag)>(src, dst, L, c->open, c->fib[fc], c->fib[fp], c->list[fp],
                                                  &c->ctr->count[fp], cap, status, true, s);
-        });
+        };
+        if (c->cfg.storage == LBMIB_FP64) lattice(double{});
+        else lattice(float{});
         c->launches++;
         spread_done = k + 1 < n && (dyn || !rep);   // the Kinematic spread needs the repulsion at X^{n+1}
         nd.Flc = tape && tape->flc && spread_done ? tape->flc + (k + 1) * tape->nodes : nullptr;

@@ -774,8 +774,8 @@ void set_wide_smem_limits(int max_n, int arcs) {
     (const void*)k_wide_dyn<S, true, true>, (const void*)k_wide_dyn<S, true, false>,                             \
         (const void*)k_wide_dyn<S, false, true>, (const void*)k_wide_kin<S, true, true>,                         \
         (const void*)k_wide_kin<S, true, false>, (const void*)k_wide_kin<S, false, true>
-    raise(cur[0], wide_smem<float>(max_n, arcs), {LBMIB_WIDE(float), LBMIB_WIDE(__half)});
-    raise(cur[1], wide_smem<double>(max_n, arcs), {LBMIB_WIDE(double), LBMIB_WIDE(f32w), LBMIB_WIDE(f16w)});
+    raise(cur[0], wide_smem<float>(max_n, arcs), {LBMIB_WIDE(float)});
+    raise(cur[1], wide_smem<double>(max_n, arcs), {LBMIB_WIDE(double), LBMIB_WIDE(f32w)});
 #undef LBMIB_WIDE
 }
 
@@ -818,14 +818,11 @@ void launch_collide_forced(const void* src, void* dst, const Lat& L, const OpenB
                                  double*, int*, int*, unsigned*, double2*, bool, cudaStream_t);
 LBMIB_INSTANTIATE_WIDE(double)
 LBMIB_INSTANTIATE_WIDE(float)
-LBMIB_INSTANTIATE_WIDE(__half)
 LBMIB_INSTANTIATE_WIDE(f32w)
-LBMIB_INSTANTIATE_WIDE(f16w)
 #define LBMIB_INSTANTIATE_FORCED(S)                                                                            \
     template void launch_collide_forced<S>(const void*, void*, const Lat&, const OpenBC&, const double*, double*, \
                                            const int*, const int*, int, unsigned*, bool, cudaStream_t);
 LBMIB_INSTANTIATE_FORCED(double)
 LBMIB_INSTANTIATE_FORCED(float)
-LBMIB_INSTANTIATE_FORCED(__half)
 
 }  // namespace lbmib

@@ -1,0 +1,73 @@
+"""Which kernels a step takes, by their number: the two-kernel step launches 2n + 1 kernels for
+n steps enqueued directly, the general kernels 3n + 1 (one CTA per capsule, update and next
+spread fused) or 4n; and that a context that keeps the general kernels computes what it does
+with them asked for by name."""
+import numpy as np
+import pytest
+
+import oracle as o
+from paper_1903_03356_gb300 import workloads as W
+
+pytestmark = pytest.mark.gpu
+
+N = 6
+
+
+@pytest.fixture(scope="module")
+def L():
+    torch = pytest.importorskip("torch")
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    from paper_1903_03356_gb300 import lbmib
+    return lbmib
+
+
+def rows(count, n, nx, ny, radius):
+    """`count` circles of n vertices in rows between walls."""
+    cols = int(nx // (2.0 * radius + 6.0))
+    caps = []
+    for k in range(count):
+        xy = W.circle(n, radius, (k % cols + 0.5) * nx / cols + 0.0137, 5.0 + radius + (k // cols) * (2.0 * radius + 5.0))
+        caps.append(W.Capsule(xy, 0.01, 0.001, 0.0, W.node_mass(1.0, W.signed_area(xy), n)))
+        assert xy[:, 1].max() < ny - 4.0
+    return W.Case("rows", nx, ny, 0.8, True, -0.005, 0.005, gx=1e-7, init="shear", capsules=caps)
+
+
+def launches(L, case, storage, scheme, **opts):
+    """Kernels of N steps enqueued directly."""
+    ctx = L.from_case(case, storage=storage)
+    ctx.set_option(L.OPT_GRAPHS, 0)
+    for k, v in opts.items():
+        ctx.set_option(getattr(L, k), v)
+    n0 = ctx.launch_count
+    ctx.step(N, scheme)
+    count = ctx.launch_count - n0
+    ctx.sync()
+    ctx.close()
+    return count
+
+
+TWO, FUSED, SPLIT = 2 * N + 1, 3 * N + 1, 4 * N
+
+
+@pytest.mark.parametrize("scheme", [o.KINEMATIC, o.DYNAMIC])
+@pytest.mark.parametrize("count, n, nx, ny, radius", [(1, 300, 160, 120, 30.0), (60, 128, 900, 500, 16.0)])
+@pytest.mark.parametrize("ib_fp64", [0, 1])
+def test_fp16_storage_keeps_the_general_kernels(L, scheme, count, n, nx, ny, radius, ib_fp64):
+    case = rows(count, n, nx, ny, radius)
+    assert launches(L, case, "fp16", scheme, OPT_IB_FP64=ib_fp64) == SPLIT
+
+
+def test_fp16_results_are_those_of_the_general_kernels(L):
+    # FP64 interpolations: the general kernels then add their shares in double and repeat
+    # themselves; a share rounded differently at every node parts FP16 populations by 1e-4
+    case = rows(60, 128, 900, 500, 16.0)
+    out = []
+    for overlap in (-1, 1):
+        ctx = L.from_case(case, storage="fp16")
+        ctx.set_option(L.OPT_IB_FP64, 1)
+        ctx.set_option(L.OPT_OVERLAP, overlap)
+        ctx.step(40, o.DYNAMIC)
+        ctx.sync()
+        out.append(ctx.field_view(L.FIELD_POPULATIONS)[:, :, :case.nx].double().cpu().numpy())   # less the rest weights
+    assert np.linalg.norm(out[0] - out[1]) < 1e-5 * np.linalg.norm(out[1])
