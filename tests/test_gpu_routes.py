@@ -71,3 +71,15 @@ def test_fp16_results_are_those_of_the_general_kernels(L):
         ctx.sync()
         out.append(ctx.field_view(L.FIELD_POPULATIONS)[:, :, :case.nx].double().cpu().numpy())   # less the rest weights
     assert np.linalg.norm(out[0] - out[1]) < 1e-5 * np.linalg.norm(out[1])
+
+
+@pytest.mark.parametrize("scheme", [o.KINEMATIC, o.DYNAMIC])
+@pytest.mark.parametrize("storage, ib_fp64, overlap", [("fp16", 0, False), ("fp16", 1, True), ("fp32", 0, True)])
+def test_fused_fp16_steps_stay_on_the_context_stream(L, scheme, storage, ib_fp64, overlap):
+    # the node update is timed only where it shares the lattice kernel's stream
+    case = rows(160, 40, 700, 400, 8.0)
+    ctx = L.from_case(case, storage=storage)
+    ctx.set_option(L.OPT_IB_FP64, ib_fp64)
+    ctx.set_option(L.OPT_TIMING, 1)
+    ctx.step(N, scheme)
+    assert ctx.ib_kernel_time()[2] == (0 if overlap else N)
