@@ -1231,7 +1231,7 @@ lbmib_status tape_forward(lbmib_ctx* c, lbmib_scheme scheme, int len, char* w, c
     double2* tX = (double2*)(w + a.tape_X);
     LBMIB_CUDA(c, cudaMemcpyAsync(tape, c->pops[c->cur], pbytes, cudaMemcpyDeviceToDevice, s));
     LBMIB_CUDA(c, cudaMemcpyAsync(w + a.age0, c->nd.age, M * sizeof(int), cudaMemcpyDeviceToDevice, s));
-    if (wide(c)) {
+    if (wide(c, scheme)) {
         const WideTape t{tape, a.pb, M, tX, scheme == LBMIB_DYNAMIC ? (double2*)(w + a.tape_flc) : nullptr};
         LBMIB_CUDA(c, cudaMemcpyAsync(tX, c->nd.X, M * sizeof(double2), cudaMemcpyDeviceToDevice, s));
         int cur = 0;

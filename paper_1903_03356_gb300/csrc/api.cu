@@ -177,6 +177,13 @@ void with_ib_storage(const lbmib_ctx* c, F&& f) {
 //  - up to kWideVerts vertices (a quarter of that where the interpolations are in FP64, whose
 //    pipe the nine-lane gathers would fill) the gathers of every support node are cheaper
 //    than the tiles' chain;
+//  - with FP64 interpolations the FP64 work of a multiprocessor decides. Up to kWideAlone
+//    CTAs each has one to itself, and with FP64 storage, whose lattice update keeps the tiled
+//    kernels waiting, two kernels always win (us per step, two kernels : tiled, 8 x 512
+//    vertices Dynamic 110 : 142, 15 x 400 99 : 143); over FP32 storage in the Dynamic scheme
+//    up to 48 vertices per CTA (8 x 384 75 : 78, but 8 x 512 96 : 89). Beyond, two CTAs share
+//    one: Dynamic FP64 up to 32 vertices per CTA (32 x 256 123 : 153, 16 x 384 150 : 142), over
+//    FP32 up to 16 (32 x 128 61 : 69; 16 x 256 96 : 73, Kinematic 45 : 43);
 //  - in single precision only where a tiled arc is longer than a warp: shorter arcs add
 //    their float shares in a fixed order, so that a tiled run repeats bit for bit, and
 //    positions, which add up every step's rounding, would part from it by 1e-9 in 200 steps;
@@ -185,15 +192,24 @@ void with_ib_storage(const lbmib_ctx* c, F&& f) {
 //    few thousand by such a step, and after 40 steps with 60 capsules on 900 x 500 the
 //    populations of the two paths were 1.3e-4 of their norm apart (the tiled kernels repeat
 //    themselves to 1e-6, and with FP64 interpolations bit for bit).
-bool wide(const lbmib_ctx* c) {
+bool wide(const lbmib_ctx* c, lbmib_scheme scheme) {
     constexpr long long kWideNodes = 1 << 20, kWideVerts = 32768;
-    const bool fp64 = c->cfg.storage == LBMIB_FP64 || c->ib_fp64;
+    const bool fp64 = c->cfg.storage == LBMIB_FP64 || c->ib_fp64, dyn = scheme == LBMIB_DYNAMIC;
     if (c->caps.empty() || c->nrigid > 0 || !c->fuse_ib || c->timing || c->overlap != -1 || c->arcs_opt != 0 ||
         c->cfg.storage == LBMIB_FP16)
         return false;
-    if (!fp64 && (c->max_n + c->arcs - 1) / c->arcs <= 32) return false;
+    const int ncaps = (int)c->caps.size(), arcs = wide_arcs(c->max_n, ncaps, c->sms > 0 ? c->sms : 1);
+    if (fp64) {
+        const int per_cta = (c->max_n + arcs - 1) / arcs;
+        int most = c->max_n;   // vertices per CTA
+        if (c->cfg.storage != LBMIB_FP64) most = ncaps * arcs > kWideAlone ? 16 : (dyn ? 48 : most);
+        else if (dyn && ncaps * arcs > kWideAlone) most = 32;
+        if (per_cta > most) return false;
+    } else if ((c->max_n + c->arcs - 1) / c->arcs <= 32) {
+        return false;
+    }
     return (long long)c->cfg.nx * c->cfg.ny <= kWideNodes && c->nd.count <= (fp64 ? kWideVerts / 4 : kWideVerts) &&
-           wide_fits(c->max_n, wide_arcs(c->max_n, (int)c->caps.size(), c->sms > 0 ? c->sms : 1));
+           wide_fits(c->max_n, arcs);
 }
 
 // Enqueue n steps of one scheme on stream s in the two-kernel form:
@@ -394,7 +410,7 @@ bool enqueue_step(lbmib_ctx* c, lbmib_scheme scheme, int& cur, int& cur_fib, cud
 // Enqueue n steps of one scheme on stream s, fusing each Dynamic update with the next
 // step's force and spread where fusable.
 void enqueue_steps(lbmib_ctx* c, lbmib_scheme scheme, long long n, int& cur, int& cur_fib, cudaStream_t s, bool timed) {
-    if (wide(c)) {
+    if (wide(c, scheme)) {
         enqueue_wide(c, scheme, n, cur, cur_fib, s, nullptr);
         return;
     }

@@ -134,7 +134,8 @@ void drop_graphs(lbmib_ctx* c);
 // by fork_ib() and join_ib() on s.
 bool enqueue_step(lbmib_ctx* c, lbmib_scheme scheme, int& cur, int& cur_fib, cudaStream_t s, bool timed,
                   bool spread_done = false, bool fuse_next = false);
-// The two-kernel step (wide.cu): whether the context's steps take it, and n such steps.
+// The two-kernel step (wide.cu): whether the context's steps of a scheme take it, and n such
+// steps.
 // The adjoint's tape: population buffer k at pops + k * stride, the positions before step k
 // at X + k * nodes, c_l F_l of step k's Dynamic spread at flc + k * nodes (may be null).
 struct WideTape {
@@ -143,7 +144,7 @@ struct WideTape {
     double2* X;
     double2* flc;
 };
-bool wide(const lbmib_ctx* c);
+bool wide(const lbmib_ctx* c, lbmib_scheme scheme);
 void enqueue_wide(lbmib_ctx* c, lbmib_scheme scheme, long long n, int& cur, int& cur_fib, cudaStream_t s,
                   const WideTape* tape);
 void fork_ib(lbmib_ctx* c, cudaStream_t s);

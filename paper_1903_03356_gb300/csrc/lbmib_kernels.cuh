@@ -122,6 +122,7 @@ void launch_interp_points(const void* src, const Lat& L, const double* fib, cons
 // list's length (0 without a spread); tape (may be null): X^{n+1} of every vertex; pdl:
 // may start before the kernel before it has finished (that kernel writes no vertex data).
 int wide_arcs(int max_n, int ncaps, int sms);
+constexpr int kWideAlone = 120;        // CTAs that find a multiprocessor each (wide.cu)
 bool wide_fits(int max_n, int arcs);   // the arcs' staged vertices fit the shared memory of a CTA
 void set_wide_smem_limits(int max_n, int arcs);
 template <typename S>

@@ -755,6 +755,14 @@ int wide_arcs(int max_n, int ncaps, int sms) {
     return std::max(1, std::min({kMaxArcs, (max_n + 15) / 16, 2 * sms / std::max(ncaps, 1)}));
 }
 
+// FP64 interpolations: two CTAs on one multiprocessor share its FP64 pipe and take twice as
+// long, and beside the lattice kernel's last CTAs the scheduler does put two clusters onto the
+// same multiprocessors while others are idle (8 rings of 512 vertices, Dynamic 183 us per step,
+// alone 110; 2 rings with the repulsion 184 and 105). Asking for more than half of the shared
+// memory keeps a CTA alone. Only while all find a place: fifteen clusters of eight do, with
+// sixteen a second round follows (16 x 128 vertices 64 us, sharing 56).
+constexpr size_t kAloneBytes = 116 * 1024;
+
 bool wide_fits(int max_n, int arcs) { return wide_smem<double>(max_n, arcs) <= 200 * 1024; }
 
 // As set_capsule_smem_limits: raised, never lowered, for the largest rings seen.
@@ -775,7 +783,7 @@ void set_wide_smem_limits(int max_n, int arcs) {
         (const void*)k_wide_dyn<S, false, true>, (const void*)k_wide_kin<S, true, true>,                         \
         (const void*)k_wide_kin<S, true, false>, (const void*)k_wide_kin<S, false, true>
     raise(cur[0], wide_smem<float>(max_n, arcs), {LBMIB_WIDE(float)});
-    raise(cur[1], wide_smem<double>(max_n, arcs), {LBMIB_WIDE(double), LBMIB_WIDE(f32w)});
+    raise(cur[1], std::max(wide_smem<double>(max_n, arcs), kAloneBytes), {LBMIB_WIDE(double), LBMIB_WIDE(f32w)});
 #undef LBMIB_WIDE
 }
 
@@ -785,7 +793,8 @@ void launch_wide(bool dynamic, bool upd, bool spr, const void* pops, const Lat& 
                  bool pdl, cudaStream_t s) {
     using C = typename St<S>::C;
     const WideIO io{fib_n, fib, list, count, status, tape};
-    const size_t sh = wide_smem<C>(max_n, arcs);
+    size_t sh = wide_smem<C>(max_n, arcs);
+    if (sizeof(C) == 8 && ncaps * arcs <= kWideAlone) sh = std::max(sh, kAloneBytes);
     // a warp for every three points of the larger sampling pass
     const int m = (max_n + arcs - 1) / arcs, pts = dynamic && upd ? 2 * (m + 1) : m;
     const int threads = std::max(128, std::min(wide_threads<S>(), (pts + 2) / 3 * 32));

@@ -83,3 +83,34 @@ def test_fused_fp16_steps_stay_on_the_context_stream(L, scheme, storage, ib_fp64
     ctx.set_option(L.OPT_TIMING, 1)
     ctx.step(N, scheme)
     assert ctx.ib_kernel_time()[2] == (0 if overlap else N)
+
+
+# (count, n, nx, ny, radius): per CTA 16, 48, 50, 64 and 32 vertices in 8 CTAs per ring, the CTAs
+# up to 120 and beyond (4 per ring with 64 rings of 128)
+SIZES = {"8x384": (8, 384, 500, 160, 20.0), "8x400": (8, 400, 500, 160, 20.0), "2x512": (2, 512, 240, 100, 30.0),
+         "15x400": (15, 400, 700, 200, 20.0), "16x384": (16, 384, 700, 200, 20.0), "16x256": (16, 256, 700, 200, 20.0),
+         "16x128": (16, 128, 700, 200, 20.0), "64x128": (64, 128, 600, 300, 12.0)}
+
+
+@pytest.mark.parametrize("storage, ib_fp64, scheme, two", [
+    ("fp64", 0, o.DYNAMIC, {"8x384", "8x400", "2x512", "15x400", "16x256", "16x128", "64x128"}),
+    ("fp64", 0, o.KINEMATIC, set(SIZES)),
+    ("fp32", 1, o.DYNAMIC, {"8x384", "16x128"}),
+    ("fp32", 1, o.KINEMATIC, {"8x384", "8x400", "2x512", "15x400", "16x128"})])
+def test_two_kernel_lines_with_fp64_interpolations(L, storage, ib_fp64, scheme, two):
+    for name, size in SIZES.items():
+        count = launches(L, rows(*size), storage, scheme, OPT_IB_FP64=ib_fp64)
+        assert (count == TWO) == (name in two), (name, count)
+
+
+@pytest.mark.parametrize("scheme", [o.KINEMATIC, o.DYNAMIC])
+@pytest.mark.parametrize("size", ["2x512", "15x400", "16x256"])
+def test_fp64_ctas_alone_and_shared_against_the_general_kernels(L, scheme, size):
+    case = rows(*SIZES[size])
+    a, b = L.from_case(case, storage="fp64"), L.from_case(case, storage="fp64")
+    b.set_option(L.OPT_OVERLAP, 1)
+    for ctx in (a, b):
+        ctx.step(12, scheme)
+    np.testing.assert_allclose(a.read_populations(), b.read_populations(), rtol=0, atol=1e-12)
+    for k in range(len(case.capsules)):
+        np.testing.assert_allclose(a.read_capsule(k)[0], b.read_capsule(k)[0], rtol=0, atol=1e-11)
