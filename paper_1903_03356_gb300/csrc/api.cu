@@ -187,6 +187,11 @@ void with_ib_storage(const lbmib_ctx* c, F&& f) {
 //  - in single precision only where a tiled arc is longer than a warp: shorter arcs add
 //    their float shares in a fixed order, so that a tiled run repeats bit for bit, and
 //    positions, which add up every step's rounding, would part from it by 1e-9 in 200 steps;
+//    and only up to one capsule per multiprocessor: with more, the tiled kernels have a CTA for
+//    each, fuse update and spread and run beside the lattice kernel, where a CTA here goes
+//    through its ring in rounds and several of them queue for a multiprocessor (Dynamic, two
+//    kernels : tiled, 152 x 144 vertices 33.4 : 38.4, 160 x 128 37.1 : 31.8, 400 x 64 37.9 : 27.2,
+//    800 x 40 60.8 : 27.7);
 //  - never with FP16 storage: it rounds a population of 1e-2 to 5e-6, so a force that differs in
 //    its last place, as the shares of the two paths do at every node, moves one population in a
 //    few thousand by such a step, and after 40 steps with 60 capsules on 900 x 500 the
@@ -205,7 +210,7 @@ bool wide(const lbmib_ctx* c, lbmib_scheme scheme) {
         if (c->cfg.storage != LBMIB_FP64) most = ncaps * arcs > kWideAlone ? 16 : (dyn ? 48 : most);
         else if (dyn && ncaps * arcs > kWideAlone) most = 32;
         if (per_cta > most) return false;
-    } else if ((c->max_n + c->arcs - 1) / c->arcs <= 32) {
+    } else if ((c->max_n + c->arcs - 1) / c->arcs <= 32 || ncaps > c->sms) {
         return false;
     }
     return (long long)c->cfg.nx * c->cfg.ny <= kWideNodes && c->nd.count <= (fp64 ? kWideVerts / 4 : kWideVerts) &&

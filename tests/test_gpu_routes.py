@@ -114,3 +114,13 @@ def test_fp64_ctas_alone_and_shared_against_the_general_kernels(L, scheme, size)
     np.testing.assert_allclose(a.read_populations(), b.read_populations(), rtol=0, atol=1e-12)
     for k in range(len(case.capsules)):
         np.testing.assert_allclose(a.read_capsule(k)[0], b.read_capsule(k)[0], rtol=0, atol=1e-11)
+
+
+@pytest.mark.parametrize("scheme", [o.KINEMATIC, o.DYNAMIC])
+def test_two_kernel_lines_in_single_precision(L, scheme):
+    for size, count in {(1, 256, 160, 120, 30.0): SPLIT, (1, 257, 160, 120, 30.0): TWO,
+                        (60, 64, 700, 300, 10.0): SPLIT, (60, 65, 700, 300, 10.0): TWO,
+                        (152, 33, 700, 300, 6.0): TWO, (152, 32, 700, 300, 6.0): FUSED,
+                        (153, 33, 700, 300, 6.0): FUSED, (400, 64, 900, 700, 10.0): FUSED,
+                        (2, 300, 1024, 1024, 30.0): TWO, (2, 300, 1024, 1025, 30.0): SPLIT}.items():
+        assert launches(L, rows(*size), "fp32", scheme) == count, size
