@@ -244,8 +244,9 @@ lbmib_status lbmib_field_ptr(lbmib_ctx* ctx, int field, void** ptr, int* pitch);
 
 /* Options (lbmib_set_option):
  *   LBMIB_OPT_GRAPHS        1 (default): replay steps from captured CUDA graphs (the
- *                           steps a call leaves over are captured when a call leaves the
- *                           same number twice in a row); 0: launch kernels directly.
+ *                           steps a call leaves over, up to 512, are captured when a
+ *                           call leaves the same number twice in a row, a few such
+ *                           numbers at a time); 0: launch kernels directly.
  *   LBMIB_OPT_TIMING        1: record CUDA events around every lattice-update launch
  *                           (forces direct launches); read with lbmib_kernel_time.
  *   LBMIB_OPT_GRAPH_STEPS   steps per captured graph (default 64; each graph opens with
@@ -331,6 +332,10 @@ lbmib_status lbmib_ib_kernel_time(lbmib_ctx* ctx, double* patch_ms, double* ib_m
 
 /* Number of kernels this context has launched (graph replays count their kernels). */
 long long lbmib_launch_count(const lbmib_ctx* ctx);
+
+/* Number of step graphs this context has captured (LBMIB_OPT_GRAPHS; the gradient's own
+ * graphs are not counted). */
+long long lbmib_capture_count(const lbmib_ctx* ctx);
 
 /* Bytes the lattice-update kernel must move per lattice update: 18 populations of the
  * storage type (9 read, 9 written). */

@@ -88,14 +88,21 @@ struct lbmib_ctx {
     cudaGraphExec_t graphs[2][2][2]{};
     int graph_len[2][2][2]{};
     long long graph_kernels[2][2][2]{};
-    // the steps a call leaves over (fewer than graph_steps): captured when a call leaves the
-    // same number twice in a row from the same buffers, one graph per (scheme, cur, cur_fib)
+    // the steps a call leaves over (fewer than graph_steps), per (scheme, cur, cur_fib): a few
+    // captured lengths, the length the last call left and how many calls in a row left it
     struct RestGraph {
         cudaGraphExec_t exec = nullptr;
-        int len = 0, seen = 0;
-        long long kernels = 0;
+        int len = 0;
+        long long kernels = 0, used = 0;   // used: the rest call that replayed it last
     };
-    RestGraph rest[2][2][2]{};
+    struct Rest {
+        RestGraph graph[4];
+        int seen = 0, row = 0;
+    };
+    Rest rest[2][2][2]{};
+    long long rest_calls = 0;
+    bool rest_failed = false;   // a capture failed: plain launches until the graphs are dropped
+    long long captures = 0;     // step graphs captured so far
     // timing
     std::vector<std::pair<cudaEvent_t, cudaEvent_t>> ev_pool;
     size_t ev_used = 0;

@@ -89,6 +89,7 @@ _SIGS = {
     "lbmib_kernel_time": (C.c_int, [_vp, _dp, C.POINTER(C.c_longlong), C.c_int]),
     "lbmib_ib_kernel_time": (C.c_int, [_vp, _dp, _dp, C.POINTER(C.c_longlong), C.POINTER(C.c_longlong), C.c_int]),
     "lbmib_launch_count": (C.c_longlong, [_vp]),
+    "lbmib_capture_count": (C.c_longlong, [_vp]),
     "lbmib_bytes_per_update": (C.c_double, [_vp]),
     "lbmib_set_repulsion": (C.c_int, [_vp, C.c_double, C.c_double]),
     "lbmib_set_inflow": (C.c_int, [_vp, _vp, C.c_double]),
@@ -238,6 +239,10 @@ def lbmib_ib_kernel_time(h, reset: bool = False):
 
 def lbmib_launch_count(h) -> int:
     return int(_lib.lbmib_launch_count(h))
+
+
+def lbmib_capture_count(h) -> int:
+    return int(_lib.lbmib_capture_count(h))
 
 
 def lbmib_bytes_per_update(h) -> float:
@@ -506,6 +511,10 @@ class Context:
     @property
     def launch_count(self) -> int:
         return lbmib_launch_count(self.h)
+
+    @property
+    def capture_count(self) -> int:
+        return lbmib_capture_count(self.h)
 
     @property
     def bytes_per_update(self) -> float:

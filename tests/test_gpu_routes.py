@@ -124,3 +124,51 @@ def test_two_kernel_lines_in_single_precision(L, scheme):
                         (153, 33, 700, 300, 6.0): FUSED, (400, 64, 900, 700, 10.0): FUSED,
                         (2, 300, 1024, 1024, 30.0): TWO, (2, 300, 1024, 1025, 30.0): SPLIT}.items():
         assert launches(L, rows(*size), "fp32", scheme) == count, size
+
+
+def test_changing_leftovers_are_captured_a_few_times_only(L):
+    case = rows(2, 40, 200, 60, 8.0)
+    a, b = L.from_case(case, storage="fp64"), L.from_case(case, storage="fp64")
+    b.set_option(L.OPT_GRAPHS, 0)
+
+    def go(*lengths):
+        before = a.capture_count
+        for n in lengths:
+            a.step(n, o.DYNAMIC)
+            b.step(n, o.DYNAMIC)
+        return a.capture_count - before
+
+    assert go(4, 6, 4, 6, 1, 1, 1) == 0        # no length twice in a row, and single steps
+    assert go(*(4, 4, 6, 6) * 8) <= 4          # from either of the two buffer parities
+    for ctx in (a, b):
+        ctx.set_option(L.OPT_GRAPH_STEPS, 64)  # drops the graphs
+    assert go(*[n for n in range(2, 40, 2) for _ in range(2)]) == 4
+    assert go(*(40,) * 15) == 0
+    assert go(*(40,) * 3) == 1                 # left sixteen times in a row: in place of the oldest
+    assert go(*(2, 2, 2)) == 0                 # the oldest was 2
+    assert go(8, 8, 8) == 0                    # still there
+    np.testing.assert_allclose(a.read_populations(), b.read_populations(), rtol=0, atol=1e-12)
+    np.testing.assert_allclose(a.read_capsule(1)[0], b.read_capsule(1)[0], rtol=0, atol=1e-11)
+    assert b.capture_count == 0
+
+
+def test_a_captured_caller_gets_plain_launches(L):
+    import torch
+
+    case = rows(2, 40, 200, 60, 8.0)
+    s = torch.cuda.Stream()
+    a, b = L.from_case(case, storage="fp64", stream=s), L.from_case(case, storage="fp64")
+    for _ in range(3):
+        for ctx in (a, b):
+            ctx.step(4, o.DYNAMIC)
+    a.sync()
+    captured = a.capture_count
+    g = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(g, stream=s):
+        a.step(4, o.DYNAMIC)
+        a.step(4, o.DYNAMIC)
+    g.replay()
+    torch.cuda.synchronize()
+    b.step(8, o.DYNAMIC)
+    assert a.capture_count == captured
+    np.testing.assert_allclose(a.read_populations(), b.read_populations(), rtol=0, atol=1e-12)
