@@ -265,19 +265,19 @@ lbmib_status lbmib_field_ptr(lbmib_ctx* ctx, int field, void** ptr, int* pitch);
  *                           step (force and spread) and of the next step (node
  *                           update); 0: every kernel on the context stream; -1
  *                           (default): on while there are fewer than two capsules per
- *                           multiprocessor (not with FP16 storage where OPT_FUSE_IB
- *                           applies, unless OPT_IB_FP64 is on), and small contexts (up
- *                           to 2^20 nodes and 32768 vertices, with FP64 interpolations
- *                           8192 and fewer where two of their CTAs would share a
- *                           multiprocessor; no rigid particles, no FP16 storage; with
- *                           FP32 interpolations at most a capsule per multiprocessor
- *                           and rings of more than a warp per CTA) step with two
- *                           kernels on the context stream, the node update with the
- *                           next spread and the lattice update with the force in
- *                           place, when OPT_ARCS and OPT_FUSE_IB are at their defaults
- *                           and OPT_TIMING is off. Results do not depend on it beyond
- *                           the order of sums, which with FP16 storage can move a
- *                           population by a storage step (as can two runs of one call).
+ *                           multiprocessor, and small contexts (up to 2^20 nodes and
+ *                           32768 vertices, with FP64 interpolations 8192 and fewer
+ *                           where two of their CTAs would share a multiprocessor; no
+ *                           rigid particles, no FP16 storage; with FP32 interpolations
+ *                           at most a capsule per multiprocessor and rings of more than
+ *                           a warp per CTA) step with two kernels on the context
+ *                           stream, the node update with the next spread and the
+ *                           lattice update with the force in place, when OPT_ARCS and
+ *                           OPT_FUSE_IB are at their defaults and OPT_TIMING is off.
+ *                           Results do not depend on it beyond the order of sums. That
+ *                           order is not fixed from run to run either, unless
+ *                           OPT_IB_FP64 is on, and FP16 storage turns a sum that falls
+ *                           out differently into a storage step of a population.
  *   LBMIB_OPT_ARCS          CTAs per capsule in the immersed-boundary kernels, 1..8:
  *                           each takes an even share of the ring's vertices, and the
  *                           kernels that need the enclosed area run a capsule's CTAs

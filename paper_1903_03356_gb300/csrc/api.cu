@@ -130,16 +130,15 @@ bool fusable(const lbmib_ctx* c) { return c->fuse_ib && c->arcs == 1 && c->nrigi
 // capsules to fill the GPU the IB blocks take registers and warp slots from the lattice
 // kernel, which slows by what the overlap saves. Hence the automatic setting: overlap
 // while the capsules number fewer than two per SM.
-// FP16 storage with the fused kernels keeps the context stream: the tiles' float additions
-// have no fixed order, FP16 rounding turns one that falls out differently into a whole step of
-// a population, and beside the lattice kernel more of them do. Two runs of 50 Kinematic steps
-// with 256 capsules on 2048 x 1024 differ by 4.6e-7 of the populations on one stream (twelve
-// inputs, median; 3.0e-6 at most) and by 7.2e-7 (5.5e-6) on two, which would take 33 instead
-// of 44 us per step. With FP64 interpolations the additions are double and both repeat bit
-// for bit.
+// FP16 storage overlaps as well. The tiles' float additions have no fixed order, on one stream
+// or two, and FP16 rounding turns one that falls out differently into a step of a population:
+// after 50 Kinematic steps with 256 capsules on 2048 x 1024, sixteen inputs, four runs each,
+// the mean distance of two runs' populations is 1.4e-6 of their norm with the overlap and 1.1e-6
+// without, and of either from a run of the kernels as they were before they could overlap
+// 1.4e-6, as of two such runs (with FP64 interpolations 0). The overlap makes it 33 instead of
+// 44 us per step.
 bool overlapped(const lbmib_ctx* c) {
     if (c->caps.empty() || c->overlap == 0) return false;
-    if (c->overlap == -1 && c->cfg.storage == LBMIB_FP16 && !c->ib_fp64 && fusable(c)) return false;
     return c->overlap == 1 || (int)c->caps.size() < 2 * (c->sms > 0 ? c->sms : 1);
 }
 
