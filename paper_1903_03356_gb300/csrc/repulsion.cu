@@ -37,6 +37,18 @@ __device__ __forceinline__ float warp_min(float v) {
 }
 __device__ __forceinline__ float warp_max(float v) { return -warp_min(-v); }
 
+// A ring that has drifted far through a periodic axis is rounded to float after whole periods
+// have been taken off, so that its float positions stay as fine as at home: at 5e8 they would
+// be rounded to multiples of 32, the ring's coarse cell could come out two cells off and its
+// partners not be found, or its box be reported as outgrown. The pair tests take minimum images
+// anyway. far_out: |x| >= 2^16, from the bits (a double comparison would hold the warp);
+// whole_periods out of line, for the same reason, and NaN beyond the positions that are sane.
+__device__ __forceinline__ bool far_out(double x) { return (__double2hiint(x) & 0x7fffffff) >= 0x40f00000; }
+__device__ __noinline__ double2 whole_periods(int nx, int ny, bool px, bool py, double x, double y) {
+    if (!(fabs(x) < 1e9 && fabs(y) < 1e9)) return make_double2(__longlong_as_double(-1), 0.0);
+    return make_double2(px ? nx * floor(x / nx) : 0.0, py ? ny * floor(y / ny) : 0.0);
+}
+
 // First chunk box of a capsule: chunks of different capsules never share a slot.
 __device__ __forceinline__ int first_chunk(int cap, int off) { return off / 32 + cap; }
 
@@ -48,11 +60,14 @@ __global__ void __launch_bounds__(128) k_rep_bin(Lat L, Nodes nd, int max_n, Rep
     const CapsuleParams P = nd.caps[c];
     if (P.n < 3 || P.n > max_n) return;
     const int first = first_chunk(c, P.off);
+    const double2 X0 = nd.X[P.off];
     const float inf = __int_as_float(0x7f800000);
     float4 b = make_float4(inf, inf, -inf, -inf);   // min x, min y, max x, max y
     for (int v0 = 32 * warp; v0 < P.n; v0 += 128) {
         const int v = v0 + lane;
-        const double2 X = nd.X[P.off + (v < P.n ? v : v0)];
+        double2 X = nd.X[P.off + (v < P.n ? v : v0)];
+        // (here, not before the loop: the two positions are one round trip)
+        if (far_out(X0.x) || far_out(X0.y)) X = X - whole_periods(L.nx, L.ny, !L.inflow, !L.walls, X0.x, X0.y);
         const float2 f = make_float2((float)X.x, (float)X.y);
         if (v < P.n) g.xf[P.off + v] = f;
         const float4 q = make_float4(warp_min(f.x), warp_min(f.y), warp_max(f.x), warp_max(f.y));
