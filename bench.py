@@ -408,12 +408,24 @@ def run_gpu(a):
     ctx.close()
 
 
-# FP64 instructions (DADD + DMUL + DFMA, thread level) per lattice update of the FP64
-# lattice kernel, from one ncu count (profiles/k_collide_stream_fp64_alu.md); GB300 issues
-# 2 such instructions per SM per cycle (ncu peak_sustained of the DFMA counter).
-FP64_INSTR_PER_UPDATE = 105.5
+# FP64 instructions (thread level, of the FP64 pipe) per lattice update of the FP64 lattice
+# kernel, k_collide_stream_d, from one ncu count (profiles/k_collide_stream_fp64_alu.md);
+# GB300 issues 2 such instructions per SM per cycle (ncu peak_sustained of the DFMA counter).
+FP64_INSTR_PER_UPDATE = 72.0
 FP64_INSTR_PER_SM_CYCLE = 2
 SM_COUNT = 152
+
+
+def fp64_roofline(glups, sm_mhz):
+    """The FP64 lattice kernel against the FP64 pipe's issue rate. More than the pipe can issue
+    means that the instruction count is not this kernel's: no fraction is given then."""
+    peak = FP64_INSTR_PER_SM_CYCLE * SM_COUNT * sm_mhz * 1e6 / 1e9   # G instr/s
+    r = {"bound": "alu", "unit": "G FP64 instr/s", "peak": peak,
+         "peak_source": "2 FP64 instructions per SM per cycle x 152 SMs x sampled SM clock",
+         "achieved": FP64_INSTR_PER_UPDATE * glups, "frac": FP64_INSTR_PER_UPDATE * glups / peak}
+    if r["frac"] > 1.0:
+        r.update(frac=None, error="above the pipe's rate: FP64_INSTR_PER_UPDATE does not fit this kernel")
+    return r
 
 
 def precision_run(L, dev, steps=(12, 60)):
@@ -445,13 +457,7 @@ def precision_run(L, dev, steps=(12, 60)):
             r["roofline"] = {"bound": "hbm", "achieved": achieved, "peak": hbm, "unit": "GB/s",
                              "frac": achieved / hbm, "peak_source": src}
         else:
-            mhz = clk.summary().get("sm_mhz") or 2070.0
-            peak = FP64_INSTR_PER_SM_CYCLE * SM_COUNT * mhz * 1e6 / 1e9   # G instr/s
-            r["roofline"] = {"bound": "alu", "unit": "G FP64 instr/s", "peak": peak,
-                             "peak_source": "2 FP64 instructions per SM per cycle x 152 SMs x sampled SM clock",
-                             "achieved": (FP64_INSTR_PER_UPDATE * gl if FP64_INSTR_PER_UPDATE else None)}
-            if FP64_INSTR_PER_UPDATE:
-                r["roofline"]["frac"] = r["roofline"]["achieved"] / peak
+            r["roofline"] = fp64_roofline(gl, clk.summary().get("sm_mhz") or 2070.0)
         out[storage] = r
         ctx.close()
     return out
@@ -480,14 +486,10 @@ def fp64_coupled_run(L, a, case, scheme, dev, steps=20, warmup=3):
     per = kms / max(1, kn)
     nodes = a.nx * a.ny
     gl = nodes / (per / 1e3) / 1e9
-    mhz = clk.summary().get("sm_mhz") or 2070.0
-    peak = FP64_INSTR_PER_SM_CYCLE * SM_COUNT * mhz * 1e6 / 1e9
     ctx.close()
     return {"workload": workload_name(a, case).replace(f"-{a.storage}", "-fp64"), "steps": steps,
             "ms_per_step": ms, "mlups": nodes / ms / 1e3, "lattice_kernel_ms": per, "lattice_share": per / ms,
-            "roofline": {"bound": "alu", "unit": "G FP64 instr/s", "peak": peak,
-                         "achieved": FP64_INSTR_PER_UPDATE * gl, "frac": FP64_INSTR_PER_UPDATE * gl / peak,
-                         "peak_source": "2 FP64 instructions per SM per cycle x 152 SMs x sampled SM clock"},
+            "roofline": fp64_roofline(gl, clk.summary().get("sm_mhz") or 2070.0),
             "clocks": clk.summary()}
 
 
