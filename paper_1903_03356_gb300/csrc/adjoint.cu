@@ -555,14 +555,6 @@ __global__ void __launch_bounds__(256) k_adj_lattice(const S* __restrict__ post0
     }
 }
 
-// 1 / sqrt(x) in double: the hardware's approximation (about 22 bits) and two Newton steps.
-__device__ __forceinline__ double rsqrt_newton(double x) {
-    double y;
-    asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
-    y = fma(0.5 * y, fma(-x * y, y, 1.0), y);
-    return fma(0.5 * y, fma(-x * y, y, 1.0), y);
-}
-
 // Shared memory of the kernels that call membrane_transpose: the staged ring and three more
 // double2 per vertex.
 inline size_t transpose_smem(int max_n) {

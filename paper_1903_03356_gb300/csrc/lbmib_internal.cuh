@@ -237,13 +237,25 @@ __device__ __forceinline__ void moments(const C s[9], C& drho, C& mx, C& my) {
     my = (s[2] - s[4]) + (s[5] + s[6]) - (s[7] + s[8]);
 }
 
-// Reciprocal in double: the hardware's approximation (about 23 bits) and two Newton steps
-// r <- r + r (1 - x r). Zero, infinite and NaN x give infinities or NaN.
+// Reciprocal in double: the hardware's approximation, which works on the upper 32 bits of its
+// operand and result (PTX ISA, rcp.approx.ftz.f64: about 20 bits), and two Newton steps
+// r <- r + r (1 - x r), each of which doubles them: 20, 40, then the rounding of the last fma
+// (within one unit in the last place of the correctly rounded one). Zero, infinite and NaN x
+// give infinities or NaN, subnormal ones are taken as zero.
 __device__ __forceinline__ double rcp_newton(double x) {
     double r;
     asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(r) : "d"(x));
     r = fma(r, fma(-x, r, 1.0), r);
     return fma(r, fma(-x, r, 1.0), r);
+}
+
+// 1 / sqrt(x) in double in the same way: about 20 bits and two Newton steps
+// y <- y + y (1 - x y^2) / 2 (within two units in the last place).
+__device__ __forceinline__ double rsqrt_newton(double x) {
+    double y;
+    asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
+    y = fma(0.5 * y, fma(-x * y, y, 1.0), y);
+    return fma(0.5 * y, fma(-x * y, y, 1.0), y);
 }
 
 // The collision in double with the fewest FP64 instructions: GB300 issues one per warp and
