@@ -125,11 +125,12 @@ bool fusable(const lbmib_ctx* c) { return c->fuse_ib && c->arcs == 1 && c->nrigi
 // needs both. CS(n+1) needs the patched populations only, so it runs beside U(n) and
 // FS(n+1), which read those populations and write vertices, lists and the other force
 // buffer. The lattice kernel is HBM-bound and the IB kernels FP64- and latency-bound,
-// so the two can share the GPU. Measured on GB300: with few capsules (one CTA each,
-// most SMs idle during the IB kernels) the step time drops by a third; with enough
-// capsules to fill the GPU the IB blocks take registers and warp slots from the lattice
-// kernel, which slows by what the overlap saves. Hence the automatic setting: overlap
-// while the capsules number fewer than two per SM.
+// so the two can share the GPU while the capsules are few; with more of them the IB blocks
+// take registers and warp slots from the lattice kernel, which slows by more than the overlap
+// saves. Hence the automatic setting: overlap while the capsules number fewer than two per
+// SM. 128 vertices each, FP32, Dynamic, us per step off : on, by capsules: 256 55.4 : 45.2,
+// 304 79.0 : 74.9, 400 80.0 : 75.6, 608 126 : 138, 1216 226 : 276, 4096 495 : 581, 16384
+// 1915 : 2334 (the Kinematic scheme alike).
 // FP16 storage overlaps as well. The tiles' float additions have no fixed order, on one stream
 // or two, and FP16 rounding turns one that falls out differently into a step of a population:
 // after 50 Kinematic steps with 256 capsules on 2048 x 1024, sixteen inputs, four runs each,
@@ -172,32 +173,37 @@ void with_ib_storage(const lbmib_ctx* c, F&& f) {
 }
 
 // Whether steps run as two kernels each (wide.cu): few capsules on a lattice that stays in
-// L2, with every option that asks for the other kernels at its default. Lines:
+// L2, with every option that asks for the other kernels at its default. Lines (figures: us per
+// step, two kernels : general kernels, the latter with their overlap):
 //  - up to kWideNodes the force field read in place costs less than the patch (its launch,
-//    list and claims);
+//    list and claims): FP32, 8 x 300 vertices, Dynamic 16.2 : 33.1 on 2^18 nodes, 26.5 : 38.3
+//    on 2^20, 42.2 : 55.9 on 2^21 and 68.0 : 73.9 on 2^22; the line is lower for the sake of
+//    FP64, whose lattice update hides the tiled kernels (the same 101 : 138, 212 : 225,
+//    360 : 363, 654 : 642), and of many short rings (60 x 128 19.1 : 30.6 Kinematic and
+//    35.6 : 36.6 Dynamic on 2^19, 26.4 : 40.5 and 44.7 : 42.7 on 2^20);
 //  - up to kWideVerts vertices (a quarter of that where the interpolations are in FP64, whose
 //    pipe the nine-lane gathers would fill) the gathers of every support node are cheaper
 //    than the tiles' chain;
-//  - with FP64 interpolations the FP64 work of a multiprocessor decides. Up to kWideAlone
-//    CTAs each has one to itself, and with FP64 storage, whose lattice update keeps the tiled
-//    kernels waiting, two kernels always win (us per step, two kernels : tiled, 8 x 512
-//    vertices Dynamic 110 : 142, 15 x 400 99 : 143); over FP32 storage in the Dynamic scheme
-//    up to 48 vertices per CTA (8 x 384 75 : 78, but 8 x 512 96 : 89). Beyond, two CTAs share
-//    one: Dynamic FP64 up to 32 vertices per CTA (32 x 256 123 : 153, 16 x 384 150 : 142), over
-//    FP32 up to 16 (32 x 128 61 : 69; 16 x 256 96 : 73, Kinematic 45 : 43);
+//  - with FP64 interpolations the FP64 work of a multiprocessor decides. Up to kWideAlone CTAs
+//    each has one to itself: with FP64 storage, whose lattice update keeps the tiled kernels
+//    waiting, two kernels win (8 x 512 vertices, Dynamic, 110 : 142, 15 x 400 99 : 143); over
+//    FP32 storage in the Dynamic scheme up to 48 vertices per CTA (8 x 384 75 : 78, but 8 x 512
+//    96 : 89). Beyond, two CTAs share one: Dynamic FP64 up to 32 vertices per CTA (32 x 256
+//    123 : 153, 16 x 384 150 : 142), over FP32 up to 16 (32 x 128 61 : 69; 16 x 256 96 : 73,
+//    Kinematic 45 : 43);
 //  - in single precision only where a tiled arc is longer than a warp: shorter arcs add
 //    their float shares in a fixed order, so that a tiled run repeats bit for bit, and
 //    positions, which add up every step's rounding, would part from it by 1e-9 in 200 steps;
 //    and only up to one capsule per multiprocessor: with more, the tiled kernels have a CTA for
 //    each, fuse update and spread and run beside the lattice kernel, where a CTA here goes
-//    through its ring in rounds and several of them queue for a multiprocessor (Dynamic, two
-//    kernels : tiled, 152 x 144 vertices 33.4 : 38.4, 160 x 128 37.1 : 31.8, 400 x 64 37.9 : 27.2,
-//    800 x 40 60.8 : 27.7);
-//  - never with FP16 storage: it rounds a population of 1e-2 to 5e-6, so a force that differs in
-//    its last place, as the shares of the two paths do at every node, moves one population in a
-//    few thousand by such a step, and after 40 steps with 60 capsules on 900 x 500 the
-//    populations of the two paths were 1.3e-4 of their norm apart (the tiled kernels repeat
-//    themselves to 1e-6, and with FP64 interpolations bit for bit).
+//    through its ring in rounds and several of them queue for a multiprocessor (Dynamic,
+//    152 x 144 vertices 33.4 : 38.4, 160 x 128 37.1 : 31.8, 400 x 64 37.9 : 27.2, 800 x 40
+//    60.8 : 27.7);
+//  - never with FP16 storage: it rounds a population of 1e-2 to 5e-6, so that a force that
+//    differs in its last place, as the shares of the two paths do at every node, now and then
+//    moves one by such a step: after 40 steps with 60 capsules on 900 x 500 the populations of
+//    the two paths were 1.3e-4 of their norm apart (the tiled kernels repeat themselves to 1e-6,
+//    and with FP64 interpolations bit for bit).
 bool wide(const lbmib_ctx* c, lbmib_scheme scheme) {
     constexpr long long kWideNodes = 1 << 20, kWideVerts = 32768;
     const bool fp64 = c->cfg.storage == LBMIB_FP64 || c->ib_fp64, dyn = scheme == LBMIB_DYNAMIC;

@@ -16,7 +16,7 @@
 // on positions rounded to float, with a reach that covers the rounding; only a pair that
 // passes is decided and evaluated in double, and only a vertex with a force forms its normal.
 // (In double throughout, the two kernels took 55 of the 83 us of a step with 16 rings of
-// 1000 vertices on 1200 x 450; the step now takes 60.)
+// 1000 vertices on 1200 x 450; the step now takes 62.)
 #include "ring.cuh"
 
 namespace lbmib {
