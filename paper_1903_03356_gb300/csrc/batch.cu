@@ -19,6 +19,7 @@
 #include <cstdint>
 #include <cstring>
 #include <string>
+#include <type_traits>
 #include <vector>
 
 #include "../../include/lbmib.h"
@@ -195,10 +196,15 @@ __device__ void run_case(const BatchDev& d, int c, int nsteps, const CapSmem& sm
                 block_reduce<1, false>(area2, sm.red);
                 A = 0.5 * area2[0];
             }
-            // Single precision: the forces and support frames of all vertices first, into the slots
-            // the float terms leave unused, then one thread per (support node, vertex) for the
-            // spread: two shared float additions (compare-and-swap loops) in a thread instead
-            // of eighteen, over the whole block instead of one thread per vertex.
+            // Single precision: the forces and support frames of all vertices into the slots the
+            // float terms leave unused; then, with FP32 storage, one thread per (support node,
+            // vertex) for the spread: two shared float additions (compare-and-swap loops) in a
+            // thread instead of eighteen, over the whole block instead of one thread per vertex
+            // (512 cases x 300 steps 49.9 -> 47.1 ms). The many warps add in an order that changes
+            // from run to run, by 1e-10 of the positions in FP32; FP16 storage makes 1e-7 of it
+            // and keeps one thread per vertex, whose order does not (35.2 us per step either way,
+            // 512 cases of 64 x 64).
+            constexpr bool kByNode = std::is_same<S, float>::value;
             for (int v = threadIdx.x; v < n; v += blockDim.x) {
                 double2 F;
                 if constexpr (F32) {
@@ -211,21 +217,24 @@ __device__ void run_case(const BatchDev& d, int c, int nsteps, const CapSmem& sm
                     const bool in = support_centre(L, x, y, cx, cy);
                     centre[v] = make_int2(cx, cy);
                     reinterpret_cast<float2*>(sm.bs)[v] = make_float2((float)((double)cx - x), (float)((double)cy - y));
-                    if (t.use) ok &= in && t.holds(cx, cy);
+                    if (kByNode && t.use) ok &= in && t.holds(cx, cy);
                 } else {
                     F = node_internal_force(sm, P, v, A);
+                }
+                if constexpr (!kByNode) {
                     if (t.use) {
                         const MlsW<C> m = mls_setup<C>(L, sm.X[v].x, sm.X[v].y);
                         ok &= m.ok && t.holds(m.cx, m.cy);
                         if (t.holds(m.cx, m.cy)) {
+                            const C Fx = C(F.x), Fy = C(F.y);
 #pragma unroll
                             for (int b = 0; b < 3; b++)
 #pragma unroll
                                 for (int a = 0; a < 3; a++) {
                                     const C phi = m.phi(a, b);
                                     const int k = t.index(m.cx + a - 1, m.cy + b - 1);
-                                    atomicAdd(t.fx + k, phi * C(F.x));
-                                    atomicAdd(t.fy + k, phi * C(F.y));
+                                    atomicAdd(t.fx + k, phi * Fx);
+                                    atomicAdd(t.fy + k, phi * Fy);
                                 }
                         }
                     }
@@ -233,7 +242,7 @@ __device__ void run_case(const BatchDev& d, int c, int nsteps, const CapSmem& sm
                 if (step == nsteps - 1) d.nd.Fint[off + v] = F;
             }
             __syncthreads();
-            if constexpr (F32) {
+            if constexpr (kByNode) {
                 for (int q = threadIdx.x; q < (t.use ? 9 * n : 0); q += blockDim.x) {
                     const int k = q / n, v = q - k * n;
                     const int2 c = centre[v];
