@@ -266,14 +266,15 @@ lbmib_status lbmib_field_ptr(lbmib_ctx* ctx, int field, void** ptr, int* pitch);
  *                           update); 0: every kernel on the context stream; -1
  *                           (default): on while there are fewer than two capsules per
  *                           multiprocessor, and small contexts (up to 2^20 nodes and
- *                           32768 vertices, with FP64 interpolations 8192 and fewer
- *                           where two of their CTAs would share a multiprocessor; no
- *                           rigid particles, no FP16 storage; with FP32 interpolations
- *                           at most a capsule per multiprocessor and rings of more than
- *                           a warp per CTA) step with two kernels on the context
- *                           stream, the node update with the next spread and the
- *                           lattice update with the force in place, when OPT_ARCS and
- *                           OPT_FUSE_IB are at their defaults and OPT_TIMING is off.
+ *                           32768 vertices, 8192 with FP64 interpolations; no rigid
+ *                           particles, no FP16 storage; with FP32 interpolations at most
+ *                           a capsule per multiprocessor and rings of more than a warp
+ *                           per CTA; less where a CTA would hold many vertices, above
+ *                           all in FP64 and with vertices closer than about half a node)
+ *                           step with two kernels on the context stream, the node update
+ *                           with the next spread and the lattice update with the force
+ *                           in place, when OPT_ARCS and OPT_FUSE_IB are at their
+ *                           defaults and OPT_TIMING is off.
  *                           Results do not depend on it beyond the order of sums. That
  *                           order is not fixed from run to run either, unless
  *                           OPT_IB_FP64 is on, and FP16 storage turns a sum that falls

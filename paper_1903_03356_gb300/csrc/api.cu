@@ -184,13 +184,21 @@ void with_ib_storage(const lbmib_ctx* c, F&& f) {
 //  - up to kWideVerts vertices (a quarter of that where the interpolations are in FP64, whose
 //    pipe the nine-lane gathers would fill) the gathers of every support node are cheaper
 //    than the tiles' chain;
-//  - with FP64 interpolations the FP64 work of a multiprocessor decides. Up to kWideAlone CTAs
-//    each has one to itself: with FP64 storage, whose lattice update keeps the tiled kernels
-//    waiting, two kernels win (8 x 512 vertices, Dynamic, 110 : 142, 15 x 400 99 : 143); over
-//    FP32 storage in the Dynamic scheme up to 48 vertices per CTA (8 x 384 75 : 78, but 8 x 512
-//    96 : 89). Beyond, two CTAs share one: Dynamic FP64 up to 32 vertices per CTA (32 x 256
-//    123 : 153, 16 x 384 150 : 142), over FP32 up to 16 (32 x 128 61 : 69; 16 x 256 96 : 73,
-//    Kinematic 45 : 43);
+//  - the two kernels' time grows with the vertices of a CTA, the general ones' with the area of
+//    a tile, that is with the spacing of the vertices (nodes). Up to kWideAlone CTAs each has a
+//    multiprocessor to itself, beyond that two share one (rings x vertices at a spacing):
+//    FP64 storage, whose lattice update keeps the general kernels waiting, Dynamic, alone,
+//    1 x 1000 at 1.0 194 : 216, at 0.3 162 : 97, 1 x 512 at 0.3 90.3 : 73.5, 1 x 384 70.4 : 79.3;
+//    sharing, 32 x 256 at 1.0 141 : 215, at 0.3 102 : 97, 16 x 200 at 0.3 74.4 : 88.4, 16 x 384
+//    at 0.7 150 : 142; Kinematic at 0.3, alone, 1 x 800 61.2 : 60.3, 1 x 1000 73.9 : 66.0,
+//    sharing, 16 x 384 63.2 : 73.3, 16 x 512 84.4 : 76.9.
+//    FP64 interpolations over FP32 storage, Dynamic, alone, 1 x 384 at 0.7 74.0 : 76.5, at 0.6
+//    74.1 : 69.4, 1 x 256 at 0.3 52.7 : 55.2, sharing, 32 x 128 at 0.7 61 : 69, 16 x 256 96 : 73;
+//    Kinematic, alone, 1 x 800 at 1.0 64 : 103, 1 x 1000 78.7 : 67.5, 1 x 512 at 0.3 43.6 : 34.6,
+//    sharing, 16 x 256 at 0.7 44.7 : 42.5.
+//    Single precision: only rings of close vertices on shared multiprocessors lose, at 0.3
+//    32 x 384 37.2 : 32.4 Dynamic and 33.5 : 27.2 Kinematic (32 x 256 31.1 : 29.6 and
+//    15.1 : 25.0); at 0.5 the dense suspension of 16 x 1000 takes 62.5 : 70.0;
 //  - in single precision only where a tiled arc is longer than a warp: shorter arcs add
 //    their float shares in a fixed order, so that a tiled run repeats bit for bit, and
 //    positions, which add up every step's rounding, would part from it by 1e-9 in 200 steps;
@@ -211,15 +219,19 @@ bool wide(const lbmib_ctx* c, lbmib_scheme scheme) {
         c->cfg.storage == LBMIB_FP16)
         return false;
     const int ncaps = (int)c->caps.size(), arcs = wide_arcs(c->max_n, ncaps, c->sms > 0 ? c->sms : 1);
-    if (fp64) {
-        const int per_cta = (c->max_n + arcs - 1) / arcs;
-        int most = c->max_n;   // vertices per CTA
-        if (c->cfg.storage != LBMIB_FP64) most = ncaps * arcs > kWideAlone ? 16 : (dyn ? 48 : most);
-        else if (dyn && ncaps * arcs > kWideAlone) most = 32;
-        if (per_cta > most) return false;
-    } else if ((c->max_n + c->arcs - 1) / c->arcs <= 32 || ncaps > c->sms) {
-        return false;
+    const double spacing = c->max_arc_len / arc_slots(c->max_n, c->arcs);
+    const bool alone = ncaps * arcs <= kWideAlone, close = spacing < (fp64 ? 0.65 : 0.45);
+    int most = c->max_n;   // vertices per CTA
+    if (c->cfg.storage == LBMIB_FP64) {
+        if (dyn) most = alone ? (close ? 48 : most) : (close ? 24 : 32);
+        else if (close) most = alone ? 96 : 48;
+    } else if (fp64) {
+        most = !alone ? 16 : dyn ? (close ? 32 : 48) : (close ? 48 : 100);
+    } else {
+        if ((c->max_n + c->arcs - 1) / c->arcs <= 32 || ncaps > c->sms) return false;
+        if (close && !alone) most = dyn ? 0 : 32;
     }
+    if ((c->max_n + arcs - 1) / arcs > most) return false;
     return (long long)c->cfg.nx * c->cfg.ny <= kWideNodes && c->nd.count <= (fp64 ? kWideVerts / 4 : kWideVerts) &&
            wide_fits(c->max_n, arcs);
 }

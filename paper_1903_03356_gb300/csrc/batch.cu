@@ -201,9 +201,10 @@ __device__ void run_case(const BatchDev& d, int c, int nsteps, const CapSmem& sm
             // vertex) for the spread: two shared float additions (compare-and-swap loops) in a
             // thread instead of eighteen, over the whole block instead of one thread per vertex
             // (512 cases x 300 steps 49.9 -> 47.1 ms). The many warps add in an order that changes
-            // from run to run, by 1e-10 of the positions in FP32; FP16 storage makes 1e-7 of it
-            // and keeps one thread per vertex, whose order does not (35.2 us per step either way,
-            // 512 cases of 64 x 64).
+            // from run to run, by 1e-10 of the positions in FP32 (after 300 steps; as much as the
+            // few warps of longer rings do with one thread per vertex). FP16 storage makes 1e-7
+            // of it and keeps one thread per vertex, with which rings of up to two warps repeat
+            // bit for bit (34.5 us per step, 512 cases of 64 x 64, against 35.8).
             constexpr bool kByNode = std::is_same<S, float>::value;
             for (int v = threadIdx.x; v < n; v += blockDim.x) {
                 double2 F;

@@ -89,26 +89,32 @@ def test_fp16_runs_part_by_few_storage_steps(L, scheme):
         assert np.linalg.norm(other - out[0]) < 2.0 ** -11 / np.sqrt(100.0) * np.linalg.norm(out[0])
 
 
-# (count, n, nx, ny, radius): per CTA 16, 48, 50, 64 and 32 vertices in 8 CTAs per ring, the CTAs
-# up to 120 and beyond (4 per ring with 64 rings of 128)
-SIZES = {"8x384": (8, 384, 500, 160, 20.0), "8x400": (8, 400, 500, 160, 20.0), "2x512": (2, 512, 240, 100, 30.0),
-         "15x400": (15, 400, 700, 200, 20.0), "16x384": (16, 384, 700, 200, 20.0), "16x256": (16, 256, 700, 200, 20.0),
+# (count, n, nx, ny, radius): CTAs with a multiprocessor each (up to 120) and beyond, vertices
+# closer than 0.65 nodes and (the names with "far") farther apart
+SIZES = {"8x256": (8, 256, 500, 160, 15.0), "8x384": (8, 384, 500, 160, 20.0), "8x400": (8, 400, 500, 160, 20.0),
+         "8x384 far": (8, 384, 500, 260, 45.0), "8x400 far": (8, 400, 500, 260, 45.0),
+         "1x384": (1, 384, 120, 80, 25.0), "1x392": (1, 392, 120, 80, 25.0),
+         "2x512": (2, 512, 240, 100, 30.0), "2x512 far": (2, 512, 320, 170, 70.0),
+         "2x776": (2, 776, 240, 100, 30.0), "2x808 far": (2, 808, 500, 250, 100.0),
+         "15x400": (15, 400, 700, 200, 20.0), "16x384": (16, 384, 700, 200, 20.0), "16x400": (16, 400, 700, 200, 20.0),
+         "16x192": (16, 192, 700, 200, 15.0), "16x200": (16, 200, 700, 200, 15.0),
+         "16x256 far": (16, 256, 700, 400, 35.0), "16x264 far": (16, 264, 700, 400, 35.0),
          "16x128": (16, 128, 700, 200, 20.0), "64x128": (64, 128, 600, 300, 12.0)}
 
 
-@pytest.mark.parametrize("storage, ib_fp64, scheme, two", [
-    ("fp64", 0, o.DYNAMIC, {"8x384", "8x400", "2x512", "15x400", "16x256", "16x128", "64x128"}),
-    ("fp64", 0, o.KINEMATIC, set(SIZES)),
-    ("fp32", 1, o.DYNAMIC, {"8x384", "16x128"}),
-    ("fp32", 1, o.KINEMATIC, {"8x384", "8x400", "2x512", "15x400", "16x128"})])
-def test_two_kernel_lines_with_fp64_interpolations(L, storage, ib_fp64, scheme, two):
+@pytest.mark.parametrize("storage, ib_fp64, scheme, general", [
+    ("fp64", 0, o.DYNAMIC, {"8x400", "1x392", "2x512", "2x776", "15x400", "16x384", "16x400", "16x200", "16x264 far", "64x128"}),
+    ("fp64", 0, o.KINEMATIC, {"2x776", "16x400"}),
+    ("fp32", 1, o.DYNAMIC, set(SIZES) - {"8x256", "8x384 far", "16x128"}),
+    ("fp32", 1, o.KINEMATIC, set(SIZES) - {"8x256", "8x384", "1x384", "8x384 far", "8x400 far", "2x512 far", "16x128"})])
+def test_two_kernel_lines_with_fp64_interpolations(L, storage, ib_fp64, scheme, general):
     for name, size in SIZES.items():
         count = launches(L, rows(*size), storage, scheme, OPT_IB_FP64=ib_fp64)
-        assert (count == TWO) == (name in two), (name, count)
+        assert (count != TWO) == (name in general), (name, count)
 
 
 @pytest.mark.parametrize("scheme", [o.KINEMATIC, o.DYNAMIC])
-@pytest.mark.parametrize("size", ["2x512", "15x400", "16x256"])
+@pytest.mark.parametrize("size", ["2x512 far", "8x384", "16x256 far"])
 def test_fp64_ctas_alone_and_shared_against_the_general_kernels(L, scheme, size):
     case = rows(*SIZES[size])
     a, b = L.from_case(case, storage="fp64"), L.from_case(case, storage="fp64")
@@ -126,7 +132,11 @@ def test_two_kernel_lines_in_single_precision(L, scheme):
                         (60, 64, 700, 300, 10.0): SPLIT, (60, 65, 700, 300, 10.0): TWO,
                         (152, 33, 700, 300, 6.0): TWO, (152, 32, 700, 300, 6.0): FUSED,
                         (153, 33, 700, 300, 6.0): FUSED, (400, 64, 900, 700, 10.0): FUSED,
-                        (2, 300, 1024, 1024, 30.0): TWO, (2, 300, 1024, 1025, 30.0): SPLIT}.items():
+                        (2, 300, 1024, 1024, 30.0): TWO, (2, 300, 1024, 1025, 30.0): SPLIT,
+                        # vertices closer than 0.45 nodes, on shared multiprocessors and alone
+                        (16, 384, 700, 200, 20.0): SPLIT, (15, 384, 700, 200, 20.0): TWO,
+                        (64, 128, 600, 300, 8.0): TWO if scheme == o.KINEMATIC else SPLIT,
+                        (64, 132, 600, 300, 8.0): SPLIT}.items():
         assert launches(L, rows(*size), "fp32", scheme) == count, size
 
 
