@@ -19,6 +19,7 @@
 
 #include <algorithm>
 #include <initializer_list>
+#include <map>
 #include <mutex>
 #include <utility>
 
@@ -765,12 +766,16 @@ constexpr size_t kAloneBytes = 116 * 1024;
 
 bool wide_fits(int max_n, int arcs) { return wide_smem<double>(max_n, arcs) <= 200 * 1024; }
 
-// As set_capsule_smem_limits: raised, never lowered, for the largest rings seen.
+// As set_capsule_smem_limits: raised, never lowered, for the largest rings seen; per device,
+// since every launch with FP64 interpolations that asks for kAloneBytes needs it.
 void set_wide_smem_limits(int max_n, int arcs) {
     if (!wide_fits(max_n, arcs)) return;
     static std::mutex mu;
-    static size_t cur[2] = {48 * 1024, 48 * 1024};
+    static std::map<int, std::pair<size_t, size_t>> limits;   // device: single, double
+    int dev = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess) return;
     std::lock_guard<std::mutex> lock(mu);
+    auto& cur = limits.emplace(dev, std::make_pair(size_t(48 * 1024), size_t(48 * 1024))).first->second;
     auto raise = [&](size_t& have, size_t bytes, std::initializer_list<const void*> kernels) {
         if (bytes <= have) return;
         bool all = true;
@@ -782,8 +787,8 @@ void set_wide_smem_limits(int max_n, int arcs) {
     (const void*)k_wide_dyn<S, true, true>, (const void*)k_wide_dyn<S, true, false>,                             \
         (const void*)k_wide_dyn<S, false, true>, (const void*)k_wide_kin<S, true, true>,                         \
         (const void*)k_wide_kin<S, true, false>, (const void*)k_wide_kin<S, false, true>
-    raise(cur[0], wide_smem<float>(max_n, arcs), {LBMIB_WIDE(float)});
-    raise(cur[1], std::max(wide_smem<double>(max_n, arcs), kAloneBytes), {LBMIB_WIDE(double), LBMIB_WIDE(f32w)});
+    raise(cur.first, wide_smem<float>(max_n, arcs), {LBMIB_WIDE(float)});
+    raise(cur.second, std::max(wide_smem<double>(max_n, arcs), kAloneBytes), {LBMIB_WIDE(double), LBMIB_WIDE(f32w)});
 #undef LBMIB_WIDE
 }
 
