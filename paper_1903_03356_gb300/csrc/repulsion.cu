@@ -63,16 +63,22 @@ __global__ void __launch_bounds__(128) k_rep_bin(Lat L, Nodes nd, int max_n, Rep
     const double2 X0 = nd.X[P.off];
     const float inf = __int_as_float(0x7f800000);
     float4 b = make_float4(inf, inf, -inf, -inf);   // min x, min y, max x, max y
-    for (int v0 = 32 * warp; v0 < P.n; v0 += 128) {
-        const int v = v0 + lane;
-        double2 X = nd.X[P.off + (v < P.n ? v : v0)];
-        // (here, not before the loop: the two positions are one round trip)
-        if (far_out(X0.x) || far_out(X0.y)) X = X - whole_periods(L.nx, L.ny, !L.inflow, !L.walls, X0.x, X0.y);
-        const float2 f = make_float2((float)X.x, (float)X.y);
-        if (v < P.n) g.xf[P.off + v] = f;
-        const float4 q = make_float4(warp_min(f.x), warp_min(f.y), warp_max(f.x), warp_max(f.y));
-        if (lane == 0) g.cbox[first + v0 / 32] = q;
-        b = make_float4(fminf(b.x, q.x), fminf(b.y, q.y), fmaxf(b.z, q.z), fmaxf(b.w, q.w));
+    auto bin = [&](double2 shift, bool shifted) {
+        for (int v0 = 32 * warp; v0 < P.n; v0 += 128) {
+            const int v = v0 + lane;
+            double2 X = nd.X[P.off + (v < P.n ? v : v0)];
+            if (shifted) X = X - shift;
+            const float2 f = make_float2((float)X.x, (float)X.y);
+            if (v < P.n) g.xf[P.off + v] = f;
+            const float4 q = make_float4(warp_min(f.x), warp_min(f.y), warp_max(f.x), warp_max(f.y));
+            if (lane == 0) g.cbox[first + v0 / 32] = q;
+            b = make_float4(fminf(b.x, q.x), fminf(b.y, q.y), fmaxf(b.z, q.z), fmaxf(b.w, q.w));
+        }
+    };
+    bin(X0, false);
+    if (far_out(X0.x) || far_out(X0.y)) {   // again (the test before would be a round trip for every ring)
+        b = make_float4(inf, inf, -inf, -inf);
+        bin(whole_periods(L.nx, L.ny, !L.inflow, !L.walls, X0.x, X0.y), true);
     }
     if (lane == 0) part[warp] = b;
     __syncthreads();
