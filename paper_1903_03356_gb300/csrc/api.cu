@@ -510,8 +510,18 @@ void update_rep_grid(lbmib_ctx* c) {
     c->nd.Fpp = c->rep_rc > 0.0 ? (double2*)(c->arena + c->lay.Fpp) : nullptr;
 }
 
+// While it lives the calling thread may instantiate a graph whatever captures are under way:
+// a caller that captures a stream of its own while it steps a context on another one, in this
+// thread or (in the global mode) in any, would otherwise find its capture invalidated.
+struct RelaxedCapture {
+    cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
+    RelaxedCapture() { cudaThreadExchangeStreamCaptureMode(&mode); }
+    ~RelaxedCapture() { cudaThreadExchangeStreamCaptureMode(&mode); }
+};
+
 lbmib_status capture(lbmib_ctx* c, lbmib_scheme scheme, int cur, int cur_fib, int len, cudaGraphExec_t* out,
                      long long* kernels) {
+    const RelaxedCapture relaxed;
     LBMIB_CUDA(c, cudaStreamBeginCapture(c->cap_stream, cudaStreamCaptureModeThreadLocal));
     const long long launches = c->launches;
     fork_ib(c, c->cap_stream);

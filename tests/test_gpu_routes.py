@@ -186,3 +186,30 @@ def test_a_captured_caller_gets_plain_launches(L):
     b.step(8, o.DYNAMIC)
     assert a.capture_count == captured
     np.testing.assert_allclose(a.read_populations(), b.read_populations(), rtol=0, atol=1e-12)
+
+
+@pytest.mark.parametrize("mode", ["global", "thread_local"])
+def test_steps_beside_a_capture_of_another_stream(L, mode):
+    # a rest that becomes a graph while the caller captures a stream the context does not use
+    import torch
+
+    case = rows(2, 40, 200, 60, 8.0)
+    a, b = L.from_case(case, storage="fp64"), L.from_case(case, storage="fp64")
+    s = torch.cuda.Stream()
+    x = torch.zeros(1000, device="cuda")
+    torch.cuda.synchronize()
+    before = a.capture_count
+    g = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(g, stream=s, capture_error_mode=mode):
+        x.add_(1.0)
+        for _ in range(3):
+            a.step(6, o.DYNAMIC)
+        a.step(70, o.DYNAMIC)
+        x.add_(1.0)
+    assert a.capture_count - before == 2
+    g.replay()
+    torch.cuda.synchronize()
+    for n in (6, 6, 6, 70):
+        b.step(n, o.DYNAMIC)
+    assert (x == 2.0).all()
+    np.testing.assert_allclose(a.read_populations(), b.read_populations(), rtol=0, atol=1e-12)
